@@ -767,10 +767,11 @@ __global__ void __launch_bounds__(kThreads, 4) rr_verify_kernel(const __grid_con
 // device memory.  One producer lane per block turns the block's work items
 // into pieces: long contiguous or row-strided 16-byte-aligned runs are loaded
 // into a ring of shared-memory stages with cp.async.bulk (rows of a strided
-// run land back to back); ragged, misaligned and zero-fill work passes
-// through as metadata only.  Consumer warps wait for a stage, cast or copy it
-// to the destination with 16-byte stores, accumulate the checksum, and
-// release the stage.  Memory latency is hidden by the ring, not by registers.
+// run land back to back); elements at any other alignment are staged in the
+// 16-byte words around them (rag_async); zero-fill work passes through as
+// metadata only.  Consumer warps wait for a stage, cast or copy it to the
+// destination with 16-byte stores, accumulate the checksum, and release the
+// stage.  Memory latency is hidden by the ring, not by registers.
 //
 // Every wait is bounded: a wait that runs out sets the plan's error word,
 // lets its block's loads land, and returns (the host reports it as RR_ECUDA).
@@ -795,6 +796,13 @@ __global__ void __launch_bounds__(kThreads, 4) rr_verify_kernel(const __grid_con
 #ifndef RR_UNPACK_WARPS
 #define RR_UNPACK_WARPS 4
 #endif
+#ifndef RR_RAG_GATHER_MAX
+#define RR_RAG_GATHER_MAX 640
+#endif
+#ifndef RR_GATHER_UNROLL
+#define RR_GATHER_UNROLL 8
+#endif
+constexpr int kGatherUnroll = RR_GATHER_UNROLL;
 
 template <int MODE>
 struct BulkShape {
@@ -812,11 +820,12 @@ enum : uint16_t {
     PC_CAST = 1,      // stage holds fp32 rows -> bf16 destination
     PC_COPY = 2,      // stage holds bf16 -> destination
     PC_READ = 3,      // stage holds bf16 that is only summed (verifying unpack gaps)
-    PC_SCALAR = 4,    // element by element from global memory
+    PC_SCALAR = 4,    // element by element from global memory (a buffer's last bytes)
     PC_ZERO_VEC = 5,  // 16-byte zero stores
     PC_ZERO_SCALAR = 6,
     PC_END = 7,
-    PC_FAN = 8        // stage holds whole rows; every fan-out destination takes its slice
+    PC_FAN = 8,       // stage holds whole rows; every fan-out destination takes its slice
+    PC_RAG = 9        // stage holds the 16-byte windows around rows of any alignment
 };
 
 constexpr uint32_t kMinBulkRowBytes = 1024;
@@ -867,6 +876,10 @@ struct BulkArgs {
     // verifying unpack): its last block leaves them zero for the slot's next
     // launch.
     uint32_t reset_claims;
+    // Bytes of each source buffer, when some are not a multiple of 16 (else
+    // NULL): a window of whole 16-byte words must not reach past a buffer's end.
+    const int64_t* src_bytes;
+    uint64_t bucket_bytes;
     unsigned long long* sums_out;  // pack through a slot: checksums[b] = sums[b] at the end
     long long* result;             // verifying unpack: {n_bad, first_bad or -1}, or NULL
     const void* ptr[NPTR];
@@ -954,6 +967,246 @@ __device__ __forceinline__ void gather_async(uint32_t stage, uint32_t full_bar, 
     asm volatile("cp.async.mbarrier.arrive.shared::cta.b64 [%0];" ::"r"(full_bar) : "memory");
 }
 
+// Rows at any alignment (a run of misaligned elements is one row): each row's
+// bytes lie in a window of whole 16-byte words.  Windows land `rag_pitch`
+// apart, each row at its own shift (its source address modulo 16).  Rows of
+// RR_RAG_GATHER_MAX bytes and more come with one bulk copy each (lane l issues
+// rows l, l + 32, ...), shorter ones with the warp's 16-byte cp.async copies.
+//
+// These elements used to be read one by one from global memory by the
+// consumers, each load waited for (19.5 of 24 cycles per issue on the load,
+// DRAM at 8%).  Staged, the path is bound by HBM like the aligned one: packing
+// a 274 M-element model of odd sizes (1.65 GB moved) went from 2467 to 244 us
+// on GB300, the verifying unpack of one whose tensors and buckets differ in
+// phase from 2957 to 165 us.  The limit between the two copy forms lies where
+// they cost the same: a bulk copy takes the copy unit about 35 ns whatever its
+// size, a gather about 35 ns per 512 bytes.  One-row pack rates: rows of 144
+// bytes 660 GB/s by bulk copies and 2280 by gathers, of 514 bytes 3050 and
+// 3620, of 1002 bytes 4260 and 3430.
+__device__ __forceinline__ uint32_t rag_pitch(uint32_t row_len, uint32_t es) {
+    return (row_len * es + 31 - es) & ~15u;   // the widest window: shift 16 - es
+}
+
+__device__ __forceinline__ void rag_async(uint32_t stage, uint32_t full_bar, const Piece& p,
+                                          uint32_t lane) {
+    const uint32_t row_bytes = p.row_len * p.es, pitch = rag_pitch(p.row_len, p.es);
+    if (p.rows > 1 && row_bytes < RR_RAG_GATHER_MAX) {
+        // Short rows: the warp's 16-byte cp.async copies, counted as in gather_async.
+        const uint32_t vpr = pitch >> 4, nv = vpr * p.rows;
+        const uint32_t dq = 32 / vpr, dr = 32 - dq * vpr;
+        const uint32_t r = lane / vpr;
+        uint32_t c = lane - r * vpr;
+        const char* row = p.src + r * p.src_stride;
+        const uint64_t step = dq * p.src_stride;
+#pragma unroll kGatherUnroll
+        for (uint32_t v = lane; v < nv; v += 32) {
+            const uint32_t sh = (uint32_t)(uintptr_t)row & 15u;
+            if (16 * c < sh + row_bytes)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage + 16 * v),
+                             "l"(row - sh + 16u * c)
+                             : "memory");
+            c += dr;
+            row += step;
+            if (c >= vpr) {
+                c -= vpr;
+                row += p.src_stride;
+            }
+        }
+        asm volatile("cp.async.mbarrier.arrive.shared::cta.b64 [%0];" ::"r"(full_bar) : "memory");
+        return;
+    }
+    uint32_t bytes = 0;
+    for (uint32_t r = lane; r < p.rows; r += 32)
+        bytes += (((uint32_t)(uintptr_t)(p.src + r * p.src_stride) & 15u) + row_bytes + 15u) & ~15u;
+    bytes = __reduce_add_sync(0xFFFFFFFFu, bytes);
+    if (lane == 0)
+        asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(full_bar),
+                     "r"(bytes)
+                     : "memory");
+    __syncwarp();
+    for (uint32_t r = lane; r < p.rows; r += 32) {
+        const char* q = p.src + r * p.src_stride;
+        const uint32_t sh = (uint32_t)(uintptr_t)q & 15u;
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes "
+            "[%0], [%1], %2, [%3];" ::"r"(stage + r * pitch),
+            "l"(q - sh), "r"((sh + row_bytes + 15u) & ~15u), "r"(full_bar)
+            : "memory");
+    }
+}
+
+__device__ __forceinline__ unsigned long long rotl64(unsigned long long v, uint32_t bits) {
+    return bits ? v << bits | v >> (64 - bits) : v;
+}
+
+// The 16-byte words of a one-row window, re-cut at the destination's 16-byte
+// boundaries: W (0..3) words into the first one, and for 2-byte elements
+// `half` more.  The shift is the same for the whole run, so it is a template
+// argument (no selects per word).  Eight elements go out per store.  `rot` is
+// 8 times the byte position, in its 64-bit checksum word, of the first of
+// those elements (a rotation, since the eight bytes keep their order).
+template <class D, int ES, int W>
+__device__ __forceinline__ unsigned long long rag_vecs(const char* q, bool half, char* dst,
+                                                       uint32_t nv, uint32_t t, uint32_t T,
+                                                       uint32_t rot) {
+    unsigned long long acc = 0;
+    const uint32_t sel = half ? 0x5432u : 0x3210u;
+    const bool more = W != 0 || half;   // the last word of a vector is touched
+#pragma unroll 4
+    for (uint32_t v = t; v < nv; v += T) {
+        uint4 o;
+        if constexpr (ES == 4) {
+            uint32_t a[12];
+            const uint4 x0 = *(const uint4*)(q + 32ull * v);
+            const uint4 x1 = *(const uint4*)(q + 32ull * v + 16);
+            const uint4 x2 = W ? *(const uint4*)(q + 32ull * v + 32) : make_uint4(0, 0, 0, 0);
+            a[0] = x0.x, a[1] = x0.y, a[2] = x0.z, a[3] = x0.w;
+            a[4] = x1.x, a[5] = x1.y, a[6] = x1.z, a[7] = x1.w;
+            a[8] = x2.x, a[9] = x2.y, a[10] = x2.z, a[11] = x2.w;
+            o.x = D::f32x2(a[W], a[W + 1]);
+            o.y = D::f32x2(a[W + 2], a[W + 3]);
+            o.z = D::f32x2(a[W + 4], a[W + 5]);
+            o.w = D::f32x2(a[W + 6], a[W + 7]);
+        } else {
+            uint32_t a[8];
+            const uint4 x0 = *(const uint4*)(q + 16ull * v);
+            const uint4 x1 = more ? *(const uint4*)(q + 16ull * v + 16) : make_uint4(0, 0, 0, 0);
+            a[0] = x0.x, a[1] = x0.y, a[2] = x0.z, a[3] = x0.w;
+            a[4] = x1.x, a[5] = x1.y, a[6] = x1.z, a[7] = x1.w;
+            o.x = __byte_perm(a[W], a[W + 1], sel);
+            o.y = __byte_perm(a[W + 1], a[W + 2], sel);
+            o.z = __byte_perm(a[W + 2], a[W + 3], sel);
+            o.w = __byte_perm(a[W + 3], a[W + 4], sel);
+            o = D::bf16x8(o);
+        }
+        if (dst) st_stream(dst + 16ull * v, o);
+        acc += rotl64((unsigned long long)o.y << 32 | o.x, rot) +
+               rotl64((unsigned long long)o.w << 32 | o.z, rot);
+    }
+    return acc;
+}
+
+// One staged element as its destination bits.
+template <class D>
+__device__ __forceinline__ uint16_t rag_elem(const char* q, uint32_t es) {
+    return es == 4 ? D::f32(*(const uint32_t*)q) : D::bf16(*(const uint16_t*)q);
+}
+
+// A one-row PC_RAG piece: scalar head up to the destination's (a summed gap's:
+// the bucket's) next 16-byte boundary, 16-byte stores, scalar tail.
+template <class D>
+__device__ __forceinline__ unsigned long long rag_run(const char* st, const Piece& p, uint32_t t,
+                                                      uint32_t T) {
+    const uint32_t es = p.es;
+    const uint32_t sh = (uint32_t)(uintptr_t)p.src & 15u;
+    const uint32_t at = p.dst ? (uint32_t)(uintptr_t)p.dst : p.sum_off;
+    const uint32_t h = min(p.n, ((16u - (at & 15u)) & 15u) >> 1);
+    const uint32_t nv = (p.n - h) >> 3;
+    const uint32_t ends = p.n - 8 * nv;   // head and tail elements, at most 14
+    unsigned long long acc = 0;
+    if (t < ends) {
+        const uint32_t e = t < h ? t : t + 8 * nv;
+        const uint16_t v = rag_elem<D>(st + sh + e * es, es);
+        if (p.dst) *(uint16_t*)(p.dst + 2ull * e) = v;
+        acc = (unsigned long long)v << (8 * ((p.sum_off + 2 * e) & 7));
+    }
+    const uint32_t b = sh + h * es;
+    const char* q = st + (b & ~15u);
+    char* d = p.dst ? p.dst + 2ull * h : nullptr;
+    const uint32_t rot = 8 * ((p.sum_off + 2 * h) & 7);
+    const bool half = b & 2;
+    switch ((es == 4 ? 4 : 0) + ((b >> 2) & 3)) {
+        case 0: return acc + rag_vecs<D, 2, 0>(q, half, d, nv, t, T, rot);
+        case 1: return acc + rag_vecs<D, 2, 1>(q, half, d, nv, t, T, rot);
+        case 2: return acc + rag_vecs<D, 2, 2>(q, half, d, nv, t, T, rot);
+        case 3: return acc + rag_vecs<D, 2, 3>(q, half, d, nv, t, T, rot);
+        case 4: return acc + rag_vecs<D, 4, 0>(q, false, d, nv, t, T, rot);
+        case 5: return acc + rag_vecs<D, 4, 1>(q, false, d, nv, t, T, rot);
+        case 6: return acc + rag_vecs<D, 4, 2>(q, false, d, nv, t, T, rot);
+        default: return acc + rag_vecs<D, 4, 3>(q, false, d, nv, t, T, rot);
+    }
+}
+
+// Eight elements from byte `b` of the stage on, as a destination vector: the
+// 16-byte words that hold them, shifted by (b & 15).
+template <class D, int ES>
+__device__ __forceinline__ uint4 rag_vec(const char* st, uint32_t b) {
+    const char* q = st + (b & ~15u);
+    const uint32_t s = b & 15u;
+    const uint4 x0 = *(const uint4*)q;
+    uint4 o;
+    if constexpr (ES == 4) {
+        const uint4 x1 = *(const uint4*)(q + 16);
+        const uint4 x2 = s ? *(const uint4*)(q + 32) : make_uint4(0, 0, 0, 0);
+        const bool two = s & 8u, one = s & 4u;
+        const uint32_t a0 = two ? x0.z : x0.x, a1 = two ? x0.w : x0.y, a2 = two ? x1.x : x0.z;
+        const uint32_t a3 = two ? x1.y : x0.w, a4 = two ? x1.z : x1.x, a5 = two ? x1.w : x1.y;
+        const uint32_t a6 = two ? x2.x : x1.z, a7 = two ? x2.y : x1.w, a8 = two ? x2.z : x2.x;
+        o.x = D::f32x2(one ? a1 : a0, one ? a2 : a1);
+        o.y = D::f32x2(one ? a3 : a2, one ? a4 : a3);
+        o.z = D::f32x2(one ? a5 : a4, one ? a6 : a5);
+        o.w = D::f32x2(one ? a7 : a6, one ? a8 : a7);
+    } else {
+        const uint4 x1 = s ? *(const uint4*)(q + 16) : make_uint4(0, 0, 0, 0);
+        const bool two = s & 8u, one = s & 4u;
+        const uint32_t a0 = two ? x0.z : x0.x, a1 = two ? x0.w : x0.y, a2 = two ? x1.x : x0.z;
+        const uint32_t a3 = two ? x1.y : x0.w, a4 = two ? x1.z : x1.x, a5 = two ? x1.w : x1.y;
+        const uint32_t b0 = one ? a1 : a0, b1 = one ? a2 : a1, b2 = one ? a3 : a2;
+        const uint32_t b3 = one ? a4 : a3, b4 = one ? a5 : a4;
+        const uint32_t sel = s & 2u ? 0x5432u : 0x3210u;
+        o = D::bf16x8(make_uint4(__byte_perm(b0, b1, sel), __byte_perm(b1, b2, sel),
+                                 __byte_perm(b2, b3, sel), __byte_perm(b3, b4, sel)));
+    }
+    return o;
+}
+
+// A PC_RAG piece of several rows, back to back in the destination: the
+// destination's 16-byte vectors, each from one row's shifted words; then the
+// vectors in which a row ends, element by element (eight lanes each).
+template <class D, int ES>
+__device__ __forceinline__ unsigned long long rag_rows(const char* st, const Piece& p, uint32_t t,
+                                                       uint32_t T) {
+    const uint32_t L = p.row_len, pitch = rag_pitch(L, ES);
+    const uint32_t s0 = (uint32_t)(uintptr_t)p.src, sr = (uint32_t)p.src_stride;
+    auto at = [&](uint32_t r, uint32_t c) { return r * pitch + ((s0 + r * sr) & 15u) + c * ES; };
+    const uint32_t h = min(p.n, ((16u - ((uint32_t)(uintptr_t)p.dst & 15u)) & 15u) >> 1);
+    const uint32_t nv = (p.n - h) >> 3;
+    const uint32_t ends = p.n - 8 * nv;   // head and tail elements, at most 14
+    unsigned long long acc = 0;
+    auto elem = [&](uint32_t e) {
+        const uint32_t r = e / L;
+        const uint16_t v = rag_elem<D>(st + at(r, e - r * L), ES);
+        *(uint16_t*)(p.dst + 2ull * e) = v;
+        acc += (unsigned long long)v << (8 * ((p.sum_off + 2 * e) & 7));
+    };
+    if (t < ends) elem(t < h ? t : t + 8 * nv);
+    char* dst = p.dst + 2 * h;
+    const uint32_t dq = 8 * T / L, dr = 8 * T - dq * L;
+    uint32_t e0 = h + 8 * t, r = e0 / L, c = e0 - r * L;
+#pragma unroll 4
+    for (uint32_t v = t; v < nv; v += T) {
+        if (c + 8 <= L) {
+            const uint4 o = rag_vec<D, ES>(st, at(r, c));
+            st_stream(dst + 16ull * v, o);
+            acc += words(o);
+        }
+        c += dr;
+        r += dq;
+        if (c >= L) {
+            c -= L;
+            ++r;
+        }
+    }
+    for (uint32_t i = t; i < 8 * (p.rows - 1); i += T) {
+        const uint32_t row = i / 8 + 1, edge = row * L;   // the first element of a row
+        if (edge <= h) continue;
+        const uint32_t v = (edge - h) >> 3, e = h + 8 * v;
+        // Inside vector v, and the first row to start inside it.
+        if (e < edge && v < nv && edge - L <= e) elem(e + (i & 7));
+    }
+    return acc;
+}
+
 template <int NPTR>
 __device__ __forceinline__ char* bulk_bucket(const BulkArgs<NPTR>& a, uint32_t b, int table_base) {
     return a.bucket_stride ? a.bucket_base + (uint64_t)b * a.bucket_stride
@@ -1013,7 +1266,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
         // arrival by lane 0, made after it wrote the piece's metadata: with the
         // byte count of its bulk copies (expect_tx), or plain.  A gather's lanes
         // have each registered their cp.async copies with the barrier first.
-        enum { kMeta = 0, kBulk = 1, kGather = 2 };
+        enum { kMeta = 0, kBulk = 1, kGather = 2, kRag = 3 };
         uint32_t count = 0;   // pieces issued
         bool ok = true;
         rr_pack_item fan_mine;   // fan-out head: lane l's destination item (l < its count)
@@ -1034,6 +1287,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
             const uint32_t stage = smem_u32(stage_mem + s * kStageBytes);
             const uint32_t row_bytes = p.row_len * p.es;
             if (how == kGather) gather_async(stage, fb, p.src, p.src_stride, p.rows, row_bytes, lane);
+            if (how == kRag) rag_async(stage, fb, p, lane);
             __syncwarp();
             if (lane != 0) {
                 ++count;
@@ -1061,6 +1315,52 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                 mbar_arrive(fb);
             }
             ++count;
+        };
+        // Elements at any alignment: p.rows rows of p.row_len elements, in a
+        // buffer whose whole 16-byte words end at `end`.  Whole rows per stage
+        // where they fit, else each row in stage-sized pieces; what lies past
+        // `end` (at most 15 bytes) is read element by element.
+        auto emit_rag = [&](Piece p, const char* end) {
+            const uint32_t es = p.es, L = p.row_len, R = p.rows;
+            const uint32_t pitch = rag_pitch(L, es);
+            const char* src = p.src;
+            char* dst = p.dst;
+            const uint32_t sum_off = p.sum_off;
+            auto piece = [&](uint32_t r, uint32_t c, uint32_t rows, uint32_t len, int how) {
+                p.kind = how == kRag ? PC_RAG : PC_SCALAR;
+                p.rows = rows;
+                p.row_len = len;
+                p.n = rows * len;
+                p.src = src + r * p.src_stride + (uint64_t)c * es;
+                p.dst = dst ? dst + 2ull * ((uint64_t)r * L + c) : nullptr;
+                p.sum_off = sum_off + 2u * (r * L + c);
+                emit(p, how);
+            };
+            const uint32_t k = (uint32_t)kStageBytes / pitch;
+            const uint32_t step = ((uint32_t)kStageBytes - 16) / es & ~7u;
+            // Rows that end at or before `end`.
+            const int64_t room = end - (src + (uint64_t)L * es);
+            const uint32_t whole =
+                room < 0 ? 0 : R == 1 ? 1 : (uint32_t)min((int64_t)R, room / (int64_t)p.src_stride + 1);
+            if (k > 0) {
+                for (uint32_t r = 0; r < whole && ok; r += k)
+                    piece(r, 0, min(k, whole - r), L, kRag);
+            } else {
+                for (uint32_t r = 0; r < whole && ok; ++r)
+                    for (uint32_t c = 0; c < L && ok; c += step)
+                        piece(r, c, 1, min(step, L - c), kRag);
+            }
+            if (!ok || whole == R) return;
+            // The rows that reach past it: one, whose first part is staged, or a
+            // few shorter than 16 bytes.
+            uint32_t in = 0;
+            if (R - whole == 1) {
+                const char* last = src + whole * p.src_stride;
+                in = last < end ? (uint32_t)((end - last) / es) : 0;
+                for (uint32_t c = 0; c < in && ok; c += step)
+                    piece(whole, c, 1, min(step, in - c), kRag);
+            }
+            if (ok) piece(whole, in, R - whole, L - in, kMeta);
         };
         // Past its own range a block claims units while any are left, the next
         // claim in flight (lane 0) while the current unit is walked.
@@ -1217,16 +1517,18 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                     p.sum_off = d.dst_off;
                     emit(p, kMeta);
                 } else {
-                    p.kind = PC_SCALAR;
                     p.es = d.kind == RR_ITEM_F32_SCALAR ? 4 : 2;
                     p.src = src;
                     p.dst = dst;
                     p.rows = d.n_rows;
                     p.row_len = d.row_len;
-                    p.n = d.row_len * d.n_rows;
                     p.src_stride = (uint64_t)d.src_stride * p.es;
                     p.sum_off = d.dst_off;
-                    emit(p, kMeta);
+                    const char* end =
+                        a.src_bytes
+                            ? (const char*)a.ptr[d.src >> 48] + (a.src_bytes[d.src >> 48] & ~15ll)
+                            : (const char*)(INT64_MAX & ~15ll);
+                    emit_rag(p, end);
                 }
             } else {
                 ItemWords<rr_unpack_item> di;
@@ -1252,14 +1554,12 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                         emit(p, kBulk);
                     }
                 } else {
-                    p.kind = PC_SCALAR;
                     p.src = src;
                     p.dst = dst;
-                    p.n = d.nbytes / 2;
                     p.rows = 1;
-                    p.row_len = p.n;
+                    p.row_len = d.nbytes / 2;
                     p.sum_off = d.src_off;
-                    emit(p, kMeta);
+                    emit_rag(p, src + ((int64_t)(a.bucket_bytes & ~15ull) - (int64_t)d.src_off));
                 }
             }
         }
@@ -1346,6 +1646,17 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                     if (kSum) acc += (unsigned long long)h << (8 * ((p.sum_off + 2 * e) & 7));
                 }
                 break;
+            case PC_RAG: {
+                unsigned long long am;
+                if (MODE != 0 || p.rows == 1)
+                    am = rag_run<D>(st, p, ct, kCT);
+                else if (p.es == 4)
+                    am = rag_rows<D, 4>(st, p, ct, kCT);
+                else
+                    am = rag_rows<D, 2>(st, p, ct, kCT);
+                if (kSum) acc += am;
+                break;
+            }
             case PC_FAN:   // pack only
                 if constexpr (MODE == 0) {
                     // Units of work: each slice's 16-byte output vectors in q parts
@@ -1879,6 +2190,8 @@ rr_status launch_bulk(const rr_plan* P, Range R, const void* const* src_shards,
     a.chk = bounds_of(P);
     a.first_bucket = R.b0;
     a.n_buckets = R.b1 - R.b0;
+    a.src_bytes = P->src_whole_words ? nullptr : P->d_src_bytes;
+    a.bucket_bytes = (uint64_t)P->bucket_bytes;
     int32_t k = 0;
     if (MODE == 0) {
         a.items = P->d_pack_items;
@@ -2341,6 +2654,8 @@ rr_status rr_device_upload(rr_plan* P) {
     std::vector<int64_t> src_bytes(size_t(P->n_shards) + 1, 0), tensor_bytes;
     rr_plan_source_buffers(P, nullptr, src_bytes.data());
     for (int32_t i = 0; i < P->n_tensors; ++i) tensor_bytes.push_back(2 * P->tensor_numel[i]);
+    P->src_whole_words = std::all_of(src_bytes.begin(), src_bytes.end(),
+                                     [](int64_t b) { return b % 16 == 0; });
     cudaError_t e;
     if ((e = up((void**)&P->d_pack_items, P->pack_items.data(),
                 P->pack_items.size() * sizeof(rr_pack_item))) != cudaSuccess ||
@@ -2370,10 +2685,11 @@ rr_status rr_device_upload(rr_plan* P) {
                 P->pack_weight_prefix.size() * sizeof(unsigned long long))) != cudaSuccess ||
         (e = up((void**)&P->d_unpack_weight_prefix, P->unpack_weight_prefix.data(),
                 P->unpack_weight_prefix.size() * sizeof(unsigned long long))) != cudaSuccess ||
+        ((P->check_items || !P->src_whole_words) &&
+         (e = up((void**)&P->d_src_bytes, src_bytes.data(), src_bytes.size() * 8)) != cudaSuccess) ||
         (P->check_items &&
-         ((e = up((void**)&P->d_src_bytes, src_bytes.data(), src_bytes.size() * 8)) != cudaSuccess ||
-          (e = up((void**)&P->d_tensor_bytes, tensor_bytes.data(), tensor_bytes.size() * 8)) !=
-              cudaSuccess)) ||
+         (e = up((void**)&P->d_tensor_bytes, tensor_bytes.data(), tensor_bytes.size() * 8)) !=
+             cudaSuccess) ||
         (!P->full_items.empty() &&
          ((e = up((void**)&P->d_full_items, P->full_items.data(),
                   P->full_items.size() * sizeof(rr_pack_item))) != cudaSuccess ||

@@ -92,8 +92,10 @@ struct rr_plan {
     unsigned long long* d_unpack_weight_prefix = nullptr;
     int32_t check_items = 0;                 // kernels check every item's bounds
     int32_t pageable_ok = 0;                 // the device can read pageable host memory
-    int64_t* d_src_bytes = nullptr;          // check_items: bytes of each source buffer
-    int64_t* d_tensor_bytes = nullptr;       //              and of each destination tensor
+    bool src_whole_words = true;             // every source buffer is a multiple of 16 bytes
+    int64_t* d_src_bytes = nullptr;          // bytes of each source buffer (check_items, or a
+                                             //   buffer that is not whole 16-byte words)
+    int64_t* d_tensor_bytes = nullptr;       // check_items: bytes of each destination tensor
     rr_unpack_item* d_unpack_items = nullptr;
     uint32_t* d_unpack_block_first = nullptr;
     uint32_t* d_unpack_unit_first = nullptr;

@@ -139,7 +139,9 @@ public:
                     continue;
                 }
             }
-            const int64_t len = std::min({l - c, chunk_elems, brem, srem});
+            // Pieces end on 16-byte boundaries of the bucket, so that the next
+            // one starts without a scalar head.
+            const int64_t len = std::min({l - c, chunk_elems - boff % 16 / 2, brem, srem});
             pack_piece(es, sh, soff, fb + bl, boff, len);
             c += len;
             if (c == l) {
@@ -171,7 +173,8 @@ public:
         while (x < nbytes) {
             const int64_t pos = P->tensor_off[t] + x;
             const int64_t bl = pos / B, boff = pos - bl * B;
-            int64_t len = std::min({nbytes - x, B - boff, P->chunk_bytes});
+            // Pieces end on 16-byte boundaries of the tensor (as in pack_run).
+            int64_t len = std::min({nbytes - x, B - boff, P->chunk_bytes - x % 16});
             copy_piece(fb + bl, boff, t, x, len);
             x += len;
         }
@@ -290,12 +293,16 @@ private:
             pack_read += row_len * n_rows * (kind <= RR_ITEM_F32_SCALAR ? 4 : 2);
     }
 
-    // One row piece: scalar head up to 16-byte destination alignment, vector
-    // body when the source is then 16-byte aligned too, scalar tail.
+    // One row piece: when the source is 16-byte aligned where the destination
+    // is, a scalar head up to there, a vector body and a scalar tail; else one
+    // scalar item.
     void split3(int vec_kind, int sc_kind, int32_t es, int64_t shard, int64_t soff,
                 int64_t bucket, int64_t boff, int64_t len, bool src_free) {
         int64_t h = ((16 - boff % 16) % 16) / 2;
-        h = std::min(h, len);
+        if (len < h + 8 || !(src_free || (soff + h * es) % 16 == 0)) {
+            if (len) emit_pack(sc_kind, shard, soff, bucket, boff, len, 1, len);
+            return;
+        }
         if (h) {
             emit_pack(sc_kind, shard, soff, bucket, boff, h, 1, h);
             soff += h * es;
@@ -303,12 +310,10 @@ private:
             len -= h;
         }
         const int64_t body = len / 8 * 8;
-        if (body && (src_free || soff % 16 == 0)) {
-            emit_pack(vec_kind, shard, soff, bucket, boff, body, 1, body);
-            soff += body * es;
-            boff += 2 * body;
-            len -= body;
-        }
+        emit_pack(vec_kind, shard, soff, bucket, boff, body, 1, body);
+        soff += body * es;
+        boff += 2 * body;
+        len -= body;
         if (len) emit_pack(sc_kind, shard, soff, bucket, boff, len, 1, len);
     }
 
@@ -364,27 +369,41 @@ private:
     }
 };
 
-int64_t pack_weight(const rr_pack_item& it) {
-    const int64_t n = int64_t(it.row_len) * it.n_rows;
-    switch (it.kind) {
-        case RR_ITEM_F32_VEC: return 6 * n + kItemOverhead;
-        case RR_ITEM_F32_SCALAR: return 12 * n + kItemOverhead;
-        case RR_ITEM_BF16_VEC: return 4 * n + kItemOverhead;
-        case RR_ITEM_BF16_SCALAR: return 8 * n + kItemOverhead;
-        case RR_ITEM_FAN_F32: return 6 * n + kItemOverhead;
-        case RR_ITEM_FAN_BF16: return 4 * n + kItemOverhead;
-        case RR_ITEM_FAN_DST: return 0;
-        default: return kZeroWeight * n + kItemOverhead;
+// Balancing weights, in bytes moved.  `staged`: the bulk-copy engine runs the
+// table.  It stages elements at any alignment: a run of them moves at nearly a
+// vector item's rate (Qwen3-like odd sizes on GB300: 6650 GB/s with 1x, 6400
+// with 1.5x, 5680 with 2x), short rows at about two thirds of it (pack 256 us
+// with 1.5x, 286 us with 1x, 280 us with 2x).  The register path moves them
+// one at a time.
+struct PackWeight {
+    bool staged;
+    int64_t operator()(const rr_pack_item& it) const {
+        const int64_t n = int64_t(it.row_len) * it.n_rows;
+        const int64_t f = !staged ? 20 : it.n_rows > 1 ? 15 : 11;   // tenths of a vector item
+        switch (it.kind) {
+            case RR_ITEM_F32_VEC: return 6 * n + kItemOverhead;
+            case RR_ITEM_F32_SCALAR: return 6 * n * f / 10 + kItemOverhead;
+            case RR_ITEM_BF16_VEC: return 4 * n + kItemOverhead;
+            case RR_ITEM_BF16_SCALAR: return 4 * n * f / 10 + kItemOverhead;
+            case RR_ITEM_FAN_F32: return 6 * n + kItemOverhead;
+            case RR_ITEM_FAN_BF16: return 4 * n + kItemOverhead;
+            case RR_ITEM_FAN_DST: return 0;
+            default: return kZeroWeight * n + kItemOverhead;
+        }
     }
-}
+};
 
-int64_t unpack_weight(const rr_unpack_item& it) {
-    switch (it.kind) {
-        case RR_ITEM_COPY_VEC: return 2 * int64_t(it.nbytes) + kItemOverhead;
-        case RR_ITEM_COPY_SCALAR: return 4 * int64_t(it.nbytes) + kItemOverhead;
-        default: return int64_t(it.nbytes) + kItemOverhead;
+struct UnpackWeight {
+    bool staged;
+    int64_t operator()(const rr_unpack_item& it) const {
+        switch (it.kind) {
+            case RR_ITEM_COPY_VEC: return 2 * int64_t(it.nbytes) + kItemOverhead;
+            case RR_ITEM_COPY_SCALAR:
+                return 2 * int64_t(it.nbytes) * (staged ? 11 : 20) / 10 + kItemOverhead;
+            default: return int64_t(it.nbytes) + kItemOverhead;
+        }
     }
-}
+};
 
 // Cuts items [0, n) into `grid` contiguous ranges of roughly equal weight.
 template <class Item, class W>
@@ -753,6 +772,9 @@ std::vector<FanGroup> find_fan_groups(const rr_plan* P, const rr_dst_layout* dst
 
 void build_tables(rr_plan* P, const rr_dst_layout* dst) {
     Builder b(P);
+    const bool staged = P->engine == RR_ENGINE_AUTO;
+    const PackWeight pack_weight{staged};
+    const UnpackWeight unpack_weight{staged};
     std::vector<std::vector<int32_t>> member;
     const std::vector<FanGroup> groups = find_fan_groups(P, dst, member);
     std::vector<std::pair<size_t, size_t>> fanned;   // regular items of grouped blocks
@@ -817,13 +839,14 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
     bucket_units(P->pack_items, P->pack_bucket_first,
                  unit_weight_for(P->pack_items, P->grid_blocks, pack_weight), P->grid_blocks,
                  P->pack_unit_first, P->pack_bucket_unit, pack_weight);
-    // Summed weights: a bucket-range call splits its items over the grid by them.
+    // Summed weights: a register-path call splits its items over the grid by
+    // them (and a bulk launch of a bucket range that gets no pooled slot).
     auto prefix = [](const auto& items, std::vector<unsigned long long>& out, auto w) {
         out.assign(items.size() + 1, 0ull);
         for (size_t i = 0; i < items.size(); ++i) out[i + 1] = out[i] + uint64_t(w(items[i]));
     };
-    prefix(P->pack_items, P->pack_weight_prefix, pack_weight);
-    prefix(P->unpack_items, P->unpack_weight_prefix, unpack_weight);
+    prefix(P->pack_items, P->pack_weight_prefix, PackWeight{false});
+    prefix(P->unpack_items, P->unpack_weight_prefix, UnpackWeight{false});
 
     // Whole-sync table: the grouped blocks' plain items give way to fan-out groups.
     P->full_items.clear();
