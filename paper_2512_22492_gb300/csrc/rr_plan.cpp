@@ -52,6 +52,9 @@ constexpr int64_t kDefaultChunkBytes = 64 * 1024;
 #ifndef RR_FAN_HEAD_CHUNKS
 #define RR_FAN_HEAD_CHUNKS 32
 #endif
+#ifndef RR_FAN_HEADS_PER_BLOCK
+#define RR_FAN_HEADS_PER_BLOCK 8
+#endif
 #ifndef RR_FAN_END_PCT
 #define RR_FAN_END_PCT 80
 #endif
@@ -221,9 +224,14 @@ public:
         const int32_t es = P->es[p];
         const int64_t C = P->cols[p], B = P->bucket_bytes;
         // Heads are cut into stage-sized pieces by the kernel; this only bounds
-        // the balancing granularity (RR_FAN_HEAD_CHUNKS chunks of source per head).
-        const int64_t max_rows =
-            std::max<int64_t>(1, RR_FAN_HEAD_CHUNKS * P->chunk_bytes / (span * es));
+        // the balancing granularity: RR_FAN_HEAD_CHUNKS chunks of source per
+        // head, and on small plans at least RR_FAN_HEADS_PER_BLOCK heads' worth
+        // of source per block (a head is one block's, and cannot be split).
+        const int64_t head_bytes =
+            std::min(RR_FAN_HEAD_CHUNKS * P->chunk_bytes,
+                     std::max(P->chunk_bytes,
+                              pack_read / (RR_FAN_HEADS_PER_BLOCK * int64_t(P->grid_blocks))));
+        const int64_t max_rows = std::max<int64_t>(1, head_bytes / (span * es));
         int64_t i = 0;
         while (i < nrows) {
             const Loc at = loc(p, (row0 + i) * C + cmin);
