@@ -1062,7 +1062,7 @@ __device__ __forceinline__ unsigned long long rag_vecs(const char* q, bool half,
     unsigned long long acc = 0;
     const uint32_t sel = half ? 0x5432u : 0x3210u;
     const bool more = W != 0 || half;   // the last word of a vector is touched
-#pragma unroll 4
+#pragma unroll 2
     for (uint32_t v = t; v < nv; v += T) {
         uint4 o;
         if constexpr (ES == 4) {
@@ -1104,10 +1104,10 @@ __device__ __forceinline__ uint16_t rag_elem(const char* q, uint32_t es) {
 
 // A one-row PC_RAG piece: scalar head up to the destination's (a summed gap's:
 // the bucket's) next 16-byte boundary, 16-byte stores, scalar tail.
-template <class D>
+template <class D, int ES>
 __device__ __forceinline__ unsigned long long rag_run(const char* st, const Piece& p, uint32_t t,
                                                       uint32_t T) {
-    const uint32_t es = p.es;
+    constexpr uint32_t es = ES;
     const uint32_t sh = (uint32_t)(uintptr_t)p.src & 15u;
     const uint32_t at = p.dst ? (uint32_t)(uintptr_t)p.dst : p.sum_off;
     const uint32_t h = min(p.n, ((16u - (at & 15u)) & 15u) >> 1);
@@ -1124,16 +1124,12 @@ __device__ __forceinline__ unsigned long long rag_run(const char* st, const Piec
     const char* q = st + (b & ~15u);
     char* d = p.dst ? p.dst + 2ull * h : nullptr;
     const uint32_t rot = 8 * ((p.sum_off + 2 * h) & 7);
-    const bool half = b & 2;
-    switch ((es == 4 ? 4 : 0) + ((b >> 2) & 3)) {
-        case 0: return acc + rag_vecs<D, 2, 0>(q, half, d, nv, t, T, rot);
-        case 1: return acc + rag_vecs<D, 2, 1>(q, half, d, nv, t, T, rot);
-        case 2: return acc + rag_vecs<D, 2, 2>(q, half, d, nv, t, T, rot);
-        case 3: return acc + rag_vecs<D, 2, 3>(q, half, d, nv, t, T, rot);
-        case 4: return acc + rag_vecs<D, 4, 0>(q, false, d, nv, t, T, rot);
-        case 5: return acc + rag_vecs<D, 4, 1>(q, false, d, nv, t, T, rot);
-        case 6: return acc + rag_vecs<D, 4, 2>(q, false, d, nv, t, T, rot);
-        default: return acc + rag_vecs<D, 4, 3>(q, false, d, nv, t, T, rot);
+    const bool half = ES == 2 && (b & 2);
+    switch ((b >> 2) & 3) {
+        case 0: return acc + rag_vecs<D, ES, 0>(q, half, d, nv, t, T, rot);
+        case 1: return acc + rag_vecs<D, ES, 1>(q, half, d, nv, t, T, rot);
+        case 2: return acc + rag_vecs<D, ES, 2>(q, half, d, nv, t, T, rot);
+        default: return acc + rag_vecs<D, ES, 3>(q, half, d, nv, t, T, rot);
     }
 }
 
@@ -1193,7 +1189,7 @@ __device__ __forceinline__ unsigned long long rag_rows(const char* st, const Pie
     char* dst = p.dst + 2 * h;
     const uint32_t dq = 8 * T / L, dr = 8 * T - dq * L;
     uint32_t e0 = h + 8 * t, r = e0 / L, c = e0 - r * L;
-#pragma unroll 4
+#pragma unroll 2
     for (uint32_t v = t; v < nv; v += T) {
         if (c + 8 <= L) {
             const uint4 o = rag_vec<D, ES>(st, at(r, c));
@@ -1326,52 +1322,6 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
             }
             ++count;
         };
-        // Elements at any alignment: p.rows rows of p.row_len elements, in a
-        // buffer whose whole 16-byte words end at `end`.  Whole rows per stage
-        // where they fit, else each row in stage-sized pieces; what lies past
-        // `end` (at most 15 bytes) is read element by element.
-        auto emit_rag = [&](Piece p, const char* end) {
-            const uint32_t es = p.es, L = p.row_len, R = p.rows;
-            const uint32_t pitch = rag_pitch(L, es);
-            const char* src = p.src;
-            char* dst = p.dst;
-            const uint32_t sum_off = p.sum_off;
-            auto piece = [&](uint32_t r, uint32_t c, uint32_t rows, uint32_t len, int how) {
-                p.kind = how == kRag ? PC_RAG : PC_SCALAR;
-                p.rows = rows;
-                p.row_len = len;
-                p.n = rows * len;
-                p.src = src + r * p.src_stride + (uint64_t)c * es;
-                p.dst = dst ? dst + 2ull * ((uint64_t)r * L + c) : nullptr;
-                p.sum_off = sum_off + 2u * (r * L + c);
-                emit(p, how);
-            };
-            const uint32_t k = (uint32_t)kStageBytes / pitch;
-            const uint32_t step = ((uint32_t)kStageBytes - 16) / es & ~7u;
-            // Rows that end at or before `end`.
-            const int64_t room = end - (src + (uint64_t)L * es);
-            const uint32_t whole =
-                room < 0 ? 0 : R == 1 ? 1 : (uint32_t)min((int64_t)R, room / (int64_t)p.src_stride + 1);
-            if (k > 0) {
-                for (uint32_t r = 0; r < whole && ok; r += k)
-                    piece(r, 0, min(k, whole - r), L, kRag);
-            } else {
-                for (uint32_t r = 0; r < whole && ok; ++r)
-                    for (uint32_t c = 0; c < L && ok; c += step)
-                        piece(r, c, 1, min(step, L - c), kRag);
-            }
-            if (!ok || whole == R) return;
-            // The rows that reach past it: one, whose first part is staged, or a
-            // few shorter than 16 bytes.
-            uint32_t in = 0;
-            if (R - whole == 1) {
-                const char* last = src + whole * p.src_stride;
-                in = last < end ? (uint32_t)((end - last) / es) : 0;
-                for (uint32_t c = 0; c < in && ok; c += step)
-                    piece(whole, c, 1, min(step, in - c), kRag);
-            }
-            if (ok) piece(whole, in, R - whole, L - in, kMeta);
-        };
         // Past its own range a block claims units while any are left, the next
         // claim in flight (lane 0) while the current unit is walked.
         unsigned long long pending = 0;
@@ -1413,6 +1363,87 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
             }
             load_words(win + 32 + lane, n0, n1);
         };
+        // One-row vector items that follow one another in the same bucket (a
+        // relay puts row-parallel weights together from its ranks' pieces, row
+        // by row) share a stage: lane l copies item win + l, window after
+        // window, and the consumers see one contiguous run.  Starts at item
+        // `it` (d); returns the items taken, or 1 with nothing issued when the
+        // next one does not follow.  A stage per item left the ring nearly
+        // empty: a TP=8 -> TP=4 relay of two Qwen3-8B layers (pieces of 1 and
+        // 3 KiB, 1.85 GB moved) packed at 862 GB/s on GB300, joined at 6.76
+        // TB/s.  Items of more than half a stage are not joined: alone they
+        // keep the ring as full.
+        auto emit_joined = [&](uint32_t it, const rr_pack_item& d, uint32_t es, char* dst) {
+            const uint32_t first = d.dst_off;
+            const uint32_t cap = (uint32_t)kStageBytes / es * 2;   // destination bytes per stage
+            uint32_t end = first, taken = 0, fb = 0;
+            int s = 0;
+            for (;;) {
+                ItemWords<rr_pack_item> m;
+                m.w[0] = w0;
+                m.w[1] = w1;
+                const uint32_t my_end = m.item.dst_off + 2 * m.item.row_len;
+                const uint32_t at = it - win;
+                uint32_t before = __shfl_up_sync(0xFFFFFFFFu, my_end, 1);
+                if (lane == at) before = end;
+                const bool follows =
+                    lane >= at && win + lane < i1 && m.item.kind == d.kind &&
+                    m.item.n_rows == 1 && m.item.bucket == d.bucket && m.item.dst_off == before &&
+                    my_end - first <= cap && (!CHECK || pack_item_in(a.chk, m.item));
+                const uint32_t gap = ~(__ballot_sync(0xFFFFFFFFu, follows) >> at);
+                const uint32_t n = min(32 - at, gap ? (uint32_t)__ffs(gap) - 1 : 32u);
+                if (taken == 0) {
+                    if (n < 2) return 1u;
+                    s = (int)(count % kStages);
+                    if (count >= (uint32_t)kStages &&
+                        !__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&empty[s]),
+                                                           ((count / kStages) - 1) & 1, a.err))) {
+                        ok = false;
+                        return 1u;
+                    }
+                    fb = smem_u32(&full[s]);
+                }
+                if (n == 0) break;
+                const uint32_t last = __shfl_sync(0xFFFFFFFFu, my_end, (int)(at + n - 1));
+                if (lane == 0)
+                    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(fb),
+                                 "r"((last - end) / 2 * es)
+                                 : "memory");
+                __syncwarp();
+                if (lane >= at && lane < at + n)
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes "
+                        "[%0], [%1], %2, [%3];" ::"r"(smem_u32(stage_mem + s * kStageBytes) +
+                                                      (m.item.dst_off - first) / 2 * es),
+                        "l"((const char*)a.ptr[m.item.src >> 48] +
+                            (m.item.src & 0xFFFFFFFFFFFFull)),
+                        "r"(m.item.row_len * es), "r"(fb)
+                        : "memory");
+                end = last;
+                taken += n;
+                it += n;
+                if (at + n < 32 || it >= i1) break;
+                window_to(it);
+            }
+            __syncwarp();
+            if (lane == 0) {
+                Piece p;
+                p.src = nullptr;
+                p.dst = dst;
+                p.src_stride = 0;
+                p.n = (end - first) / 2;
+                p.rows = 1;
+                p.row_len = p.n;
+                p.sum_bucket = d.bucket;
+                p.sum_off = first;
+                p.kind = es == 4 ? PC_CAST : PC_COPY;
+                p.es = (uint16_t)es;
+                meta[s] = p;
+                mbar_arrive(fb);
+            }
+            ++count;
+            return taken;
+        };
         for (uint32_t it = i0; ok; ++it) {
             if (it >= i1) {
                 bool more = true;
@@ -1420,9 +1451,21 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                 if (!more) break;
             }
             window_to(it);
+            // Every kind of item is described here and cut into pieces by the one
+            // loop at the end (one copy of emit in the kernel: with one per kind
+            // the unpack kernels were twice as long, and Qwen3-0.6B's sync, two
+            // launches of 0.35 and 0.5 ms, took 0.2% more): R rows of L elements,
+            // whole rows k to a stage, or (k == 0) each row in steps.  Rows from
+            // `whole` on reach past a buffer's last whole 16-byte word (staged
+            // elements of any alignment only): `in` elements of the first are
+            // staged, the rest is read element by element.
             Piece p;
-            p.dst = nullptr;
-            p.src_stride = 0;
+            const char* src;
+            char* dst = nullptr;
+            uint64_t sstride = 0;
+            uint32_t R = 1, L, k = 0, step, whole, in = 0, off, fan = 0;
+            int how = kBulk;
+            const char* end = (const char*)(INT64_MAX & ~15ll);   // PC_RAG: the buffer's
             if (MODE == 0) {
                 ItemWords<rr_pack_item> di;
                 shfl_words(w0, w1, (int)(it - win), di.w[0], di.w[1]);
@@ -1432,50 +1475,20 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                         it += min(d.dst_off, i1 - 1 - it);   // and its destinations
                     continue;
                 }
-                char* dst = bulk_bucket(a, d.bucket, a.n_shards) + d.dst_off;
-                const char* src = (const char*)a.ptr[d.src >> 48] + (d.src & 0xFFFFFFFFFFFFull);
+                const bool f32 = d.kind == RR_ITEM_F32_VEC || d.kind == RR_ITEM_F32_SCALAR ||
+                                 d.kind == RR_ITEM_FAN_F32;
+                const uint32_t es = f32 ? 4 : 2;
+                src = (const char*)a.ptr[d.src >> 48] + (d.src & 0xFFFFFFFFFFFFull);
+                R = d.n_rows;
+                L = d.row_len;
+                sstride = (uint64_t)d.src_stride * es;
+                off = d.dst_off;
+                p.es = (uint16_t)es;
                 p.sum_bucket = d.bucket;
-                if (d.kind == RR_ITEM_F32_VEC || d.kind == RR_ITEM_BF16_VEC) {
-                    const uint32_t es = d.kind == RR_ITEM_F32_VEC ? 4 : 2;
-                    const uint32_t L = d.row_len, R = d.n_rows;
-                    const uint64_t sstride = (uint64_t)d.src_stride * es;
-                    p.kind = es == 4 ? PC_CAST : PC_COPY;
-                    p.es = (uint16_t)es;
-                    if (R == 1 || L * es > (uint32_t)kStageBytes) {
-                        const uint32_t step = kStageBytes / es;
-                        for (uint32_t r = 0; r < R && ok; ++r)
-                            for (uint32_t e0 = 0; e0 < L && ok; e0 += step) {
-                                p.n = min(step, L - e0);
-                                p.rows = 1;
-                                p.row_len = p.n;
-                                p.src = src + r * sstride + (uint64_t)e0 * es;
-                                p.dst = dst + 2ull * ((uint64_t)r * L + e0);
-                                p.sum_off = d.dst_off + 2u * (r * L + e0);
-                                emit(p, kBulk);
-                            }
-                    } else {
-                        // Whole rows per stage.  Rows under kMinBulkRowBytes are gathered
-                        // by the warp's 16-byte cp.async copies (one bulk copy per short
-                        // row would leave a single issuing lane the bottleneck).
-                        const int how = L * es < kMinBulkRowBytes && sstride != L * es ? kGather : kBulk;
-                        const uint32_t k = kStageBytes / (L * es);
-                        for (uint32_t r0 = 0; r0 < R && ok; r0 += k) {
-                            p.rows = min(k, R - r0);
-                            p.row_len = L;
-                            p.n = p.rows * L;
-                            p.src_stride = sstride;
-                            p.src = src + r0 * sstride;
-                            p.dst = dst + 2ull * r0 * L;
-                            p.sum_off = d.dst_off + 2u * r0 * L;
-                            emit(p, how);
-                        }
-                    }
-                } else if (d.kind == RR_ITEM_FAN_F32 || d.kind == RR_ITEM_FAN_BF16) {
+                if (d.kind == RR_ITEM_FAN_F32 || d.kind == RR_ITEM_FAN_BF16) {
                     // Whole rows of the slices' span, staged once; the destination
                     // items that follow the head are read by the consumers.
-                    const uint32_t es = d.kind == RR_ITEM_FAN_F32 ? 4 : 2;
-                    const uint32_t rb = d.row_len * es, R = d.n_rows, nd = d.dst_off;
-                    const uint64_t sstride = (uint64_t)d.src_stride * es;
+                    const uint32_t rb = L * es, nd = d.dst_off;
                     // The planner guarantees the alignments the vector paths need;
                     // a table that breaks them is refused, not run.
                     bool bad = rb > (uint32_t)kStageBytes || rb % 16 != 0 || nd > kMaxFanDst ||
@@ -1483,17 +1496,17 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                     // Lane l's destination is item it + 1 + l: in this window or
                     // the next (it - win < 32 and nd <= kMaxFanDst).
                     {
-                        const uint32_t k = it + 1 + min((uint32_t)lane, nd > 0 ? nd - 1 : 0u) - win;
+                        const uint32_t j = it + 1 + min((uint32_t)lane, nd > 0 ? nd - 1 : 0u) - win;
                         ItemWords<rr_pack_item> c, n;
-                        shfl_words(w0, w1, (int)(k & 31u), c.w[0], c.w[1]);
-                        shfl_words(n0, n1, (int)(k & 31u), n.w[0], n.w[1]);
-                        fan_mine = k < 32u ? c.item : n.item;
+                        shfl_words(w0, w1, (int)(j & 31u), c.w[0], c.w[1]);
+                        shfl_words(n0, n1, (int)(j & 31u), n.w[0], n.w[1]);
+                        fan_mine = j < 32u ? c.item : n.item;
                     }
                     if (!bad && lane < nd) {
                         const rr_pack_item f = fan_mine;
                         bad = f.kind != RR_ITEM_FAN_DST || f.row_len % 8 != 0 ||
                               f.dst_off % 16 != 0 || (f.src * es) % 16 != 0 ||
-                              f.src + f.row_len > d.row_len || f.n_rows != R ||
+                              f.src + f.row_len > L || f.n_rows != R ||
                               (CHECK && !pack_item_in(a.chk, f));
                     }
                     if (__any_sync(0xFFFFFFFFu, bad)) {
@@ -1501,44 +1514,39 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                         ok = false;
                         break;
                     }
-                    const int how = rb < kMinBulkRowBytes && sstride != rb ? kGather : kBulk;
-                    const uint32_t k = kStageBytes / rb;
+                    how = rb < kMinBulkRowBytes && sstride != rb ? kGather : kBulk;
+                    k = kStageBytes / rb;
+                    fan = nd;
                     p.kind = PC_FAN;
-                    p.es = (uint16_t)es;
-                    p.row_len = d.row_len;
-                    p.src_stride = sstride;
                     p.sum_bucket = it + 1;   // index of the first destination item
-                    p.n = nd;
-                    for (uint32_t r0 = 0; r0 < R && ok; r0 += k) {
-                        p.rows = min(k, R - r0);
-                        p.src = src + r0 * sstride;
-                        p.sum_off = r0;      // first row of this piece within the item
-                        emit(p, how);
-                    }
                     it += nd;
-                } else if (d.kind == RR_ITEM_ZERO_VEC || d.kind == RR_ITEM_ZERO_SCALAR) {
-                    p.kind = d.kind == RR_ITEM_ZERO_VEC ? PC_ZERO_VEC : PC_ZERO_SCALAR;
-                    p.dst = dst;
-                    p.n = d.row_len;
-                    p.rows = 1;
-                    p.row_len = d.row_len;
-                    p.es = 2;
-                    p.src = nullptr;
-                    p.sum_off = d.dst_off;
-                    emit(p, kMeta);
                 } else {
-                    p.es = d.kind == RR_ITEM_F32_SCALAR ? 4 : 2;
-                    p.src = src;
-                    p.dst = dst;
-                    p.rows = d.n_rows;
-                    p.row_len = d.row_len;
-                    p.src_stride = (uint64_t)d.src_stride * p.es;
-                    p.sum_off = d.dst_off;
-                    const char* end =
-                        a.src_bytes
-                            ? (const char*)a.ptr[d.src >> 48] + (a.src_bytes[d.src >> 48] & ~15ll)
-                            : (const char*)(INT64_MAX & ~15ll);
-                    emit_rag(p, end);
+                    dst = bulk_bucket(a, d.bucket, a.n_shards) + d.dst_off;
+                    if (d.kind == RR_ITEM_F32_VEC || d.kind == RR_ITEM_BF16_VEC) {
+                        p.kind = es == 4 ? PC_CAST : PC_COPY;
+                        if (R == 1 && L * es <= (uint32_t)kStageBytes / 2) {
+                            const uint32_t taken = emit_joined(it, d, es, dst);
+                            if (taken > 1 || !ok) {
+                                it += taken - 1;
+                                continue;
+                            }
+                        }
+                        // Whole rows per stage.  Rows under kMinBulkRowBytes are gathered
+                        // by the warp's 16-byte cp.async copies.
+                        if (R > 1 && L * es <= (uint32_t)kStageBytes) {
+                            if (L * es < kMinBulkRowBytes && sstride != L * es) how = kGather;
+                            k = kStageBytes / (L * es);
+                        }
+                    } else if (d.kind == RR_ITEM_ZERO_VEC || d.kind == RR_ITEM_ZERO_SCALAR) {
+                        p.kind = d.kind == RR_ITEM_ZERO_VEC ? PC_ZERO_VEC : PC_ZERO_SCALAR;
+                        R = k = 1;
+                        how = kMeta;
+                    } else {
+                        how = kRag;
+                        if (a.src_bytes)
+                            end = (const char*)a.ptr[d.src >> 48] +
+                                  (a.src_bytes[d.src >> 48] & ~15ll);
+                    }
                 }
             } else {
                 ItemWords<rr_unpack_item> di;
@@ -1547,29 +1555,67 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                 const bool read_only = d.kind == RR_ITEM_READ_VEC || d.kind == RR_ITEM_READ_SCALAR;
                 if (MODE == 1 && read_only) continue;
                 if (CHECK && !unpack_item_ok(a.chk, d)) continue;
-                const char* src = bulk_bucket(a, d.bucket, 0) + d.src_off;
-                char* dst = read_only ? nullptr : (char*)a.ptr[a.dst_base + d.tensor] + d.dst_off;
-                p.sum_bucket = d.bucket;
+                src = bulk_bucket(a, d.bucket, 0) + d.src_off;
+                if (!read_only) dst = (char*)a.ptr[a.dst_base + d.tensor] + d.dst_off;
+                L = d.nbytes / 2;
+                off = d.src_off;
                 p.es = 2;
-                if (d.kind == RR_ITEM_COPY_VEC || d.kind == RR_ITEM_READ_VEC) {
-                    p.kind = read_only ? PC_READ : PC_COPY;
-                    for (uint32_t o = 0; o < d.nbytes && ok; o += kStageBytes) {
-                        const uint32_t len = min((uint32_t)kStageBytes, d.nbytes - o);
-                        p.n = len / 2;
-                        p.rows = 1;
-                        p.row_len = p.n;
-                        p.src = src + o;
-                        p.dst = dst ? dst + o : nullptr;
-                        p.sum_off = d.src_off + o;
-                        emit(p, kBulk);
+                p.sum_bucket = d.bucket;
+                p.kind = read_only ? PC_READ : PC_COPY;
+                if (d.kind == RR_ITEM_COPY_SCALAR || d.kind == RR_ITEM_READ_SCALAR) {
+                    how = kRag;
+                    end = src + ((int64_t)(a.bucket_bytes & ~15ull) - (int64_t)d.src_off);
+                }
+            }
+            step = (uint32_t)kStageBytes / p.es;
+            whole = R;
+            if (how == kRag) {
+                p.kind = PC_RAG;
+                k = (uint32_t)kStageBytes / rag_pitch(L, p.es);
+                step = ((uint32_t)kStageBytes - 16) / p.es & ~7u;
+                // Rows that end at or before `end`; of those that do not, one has
+                // a first part that is staged, or a few are shorter than 16 bytes.
+                const int64_t room = end - (src + (uint64_t)L * p.es);
+                if (room < 0)
+                    whole = 0;
+                else if (R > 1)
+                    whole = (uint32_t)min((int64_t)R, room / (int64_t)sstride + 1);
+                if (R - whole == 1) {
+                    const char* last = src + whole * sstride;
+                    in = last < end ? (uint32_t)((end - last) / p.es) : 0;
+                }
+            }
+            p.src_stride = sstride;
+            for (uint32_t r = 0, c = 0; r < R && ok;) {
+                p.rows = 1;
+                p.row_len = min(step, L - c);
+                int h = how;
+                if (r < whole) {
+                    if (k) {
+                        p.rows = min(k, whole - r);
+                        p.row_len = L;
                     }
+                } else if (c < in) {
+                    p.row_len = min(step, in - c);
                 } else {
-                    p.src = src;
-                    p.dst = dst;
-                    p.rows = 1;
-                    p.row_len = d.nbytes / 2;
-                    p.sum_off = d.src_off;
-                    emit_rag(p, src + ((int64_t)(a.bucket_bytes & ~15ull) - (int64_t)d.src_off));
+                    p.rows = R - whole;
+                    p.row_len = L - in;
+                    p.kind = PC_SCALAR;
+                    h = kMeta;
+                }
+                p.n = p.rows * p.row_len;
+                p.src = src + r * sstride + (uint64_t)c * p.es;
+                p.dst = dst ? dst + 2ull * ((uint64_t)r * L + c) : nullptr;
+                p.sum_off = off + 2u * (r * L + c);
+                if (MODE == 0 && fan) {
+                    p.n = fan;
+                    p.sum_off = r;   // first row of this piece within the item
+                }
+                emit(p, h);
+                c += p.row_len;
+                if (c == L) {
+                    r += p.rows;
+                    c = 0;
                 }
             }
         }
@@ -1658,12 +1704,12 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                 break;
             case PC_RAG: {
                 unsigned long long am;
-                if (MODE != 0 || p.rows == 1)
-                    am = rag_run<D>(st, p, ct, kCT);
-                else if (p.es == 4)
-                    am = rag_rows<D, 4>(st, p, ct, kCT);
+                if (MODE == 0 && p.es == 4)
+                    am = p.rows == 1 ? rag_run<D, 4>(st, p, ct, kCT)
+                                     : rag_rows<D, 4>(st, p, ct, kCT);
                 else
-                    am = rag_rows<D, 2>(st, p, ct, kCT);
+                    am = MODE != 0 || p.rows == 1 ? rag_run<D, 2>(st, p, ct, kCT)
+                                                  : rag_rows<D, 2>(st, p, ct, kCT);
                 if (kSum) acc += am;
                 break;
             }
