@@ -33,13 +33,21 @@ namespace {
 thread_local std::string g_error;
 
 constexpr int64_t kDefaultChunkBytes = 64 * 1024;
-// Balancing weights (build-time overridable for tuning sweeps).  An item costs
-// about what 3 KiB of traffic do (its copy is issued and its words read by one
-// producer warp): on a relay of 1 to 3 KiB pieces the pack ran at 430, 371,
-// 338, 287, 273 and 273 us with 0, 0.5, 1, 2, 3 and 4 KiB, and plans of large
-// items the same with each.
+// Balancing weights (build-time overridable for tuning sweeps).  Beyond its
+// bytes an item costs its copies' issue, by one producer warp.  Where short
+// items make up the table (a relay's pieces of 1 to 3 KiB, RR_SHORT_ITEM bytes
+// each on average at most) that is about 3 KiB of traffic an item: such a
+// relay's pack ran at 430, 371, 338, 287, 273 and 273 us with 0, 0.5, 1, 2, 3
+// and 4 KiB.  Tables of large items with a few short ones among them run the
+// same with each, and the odd-sized one best with 1 (244 us, 250 with 3).
 #ifndef RR_ITEM_OVERHEAD
-#define RR_ITEM_OVERHEAD 3072
+#define RR_ITEM_OVERHEAD 1024
+#endif
+#ifndef RR_SHORT_ITEM_OVERHEAD
+#define RR_SHORT_ITEM_OVERHEAD 3072
+#endif
+#ifndef RR_SHORT_ITEM
+#define RR_SHORT_ITEM (16 * 1024)
 #endif
 #ifndef RR_ZERO_WEIGHT
 #define RR_ZERO_WEIGHT 2
@@ -389,18 +397,19 @@ private:
 // one at a time.
 struct PackWeight {
     bool staged;
+    int64_t overhead = kItemOverhead;
     int64_t operator()(const rr_pack_item& it) const {
         const int64_t n = int64_t(it.row_len) * it.n_rows;
         const int64_t f = !staged ? 20 : it.n_rows > 1 ? 15 : 11;   // tenths of a vector item
         switch (it.kind) {
-            case RR_ITEM_F32_VEC: return 6 * n + kItemOverhead;
-            case RR_ITEM_F32_SCALAR: return 6 * n * f / 10 + kItemOverhead;
-            case RR_ITEM_BF16_VEC: return 4 * n + kItemOverhead;
-            case RR_ITEM_BF16_SCALAR: return 4 * n * f / 10 + kItemOverhead;
-            case RR_ITEM_FAN_F32: return 6 * n + kItemOverhead;
-            case RR_ITEM_FAN_BF16: return 4 * n + kItemOverhead;
+            case RR_ITEM_F32_VEC: return 6 * n + overhead;
+            case RR_ITEM_F32_SCALAR: return 6 * n * f / 10 + overhead;
+            case RR_ITEM_BF16_VEC: return 4 * n + overhead;
+            case RR_ITEM_BF16_SCALAR: return 4 * n * f / 10 + overhead;
+            case RR_ITEM_FAN_F32: return 6 * n + overhead;
+            case RR_ITEM_FAN_BF16: return 4 * n + overhead;
             case RR_ITEM_FAN_DST: return 0;
-            default: return kZeroWeight * n + kItemOverhead;
+            default: return kZeroWeight * n + overhead;
         }
     }
 };
@@ -785,7 +794,7 @@ std::vector<FanGroup> find_fan_groups(const rr_plan* P, const rr_dst_layout* dst
 void build_tables(rr_plan* P, const rr_dst_layout* dst) {
     Builder b(P);
     const bool staged = P->engine == RR_ENGINE_AUTO;
-    const PackWeight pack_weight{staged};
+    PackWeight pack_weight{staged};
     const UnpackWeight unpack_weight{staged};
     std::vector<std::vector<int32_t>> member;
     const std::vector<FanGroup> groups = find_fan_groups(P, dst, member);
@@ -842,6 +851,14 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
         P->bucket_tensor_lo[it.bucket] = std::min(P->bucket_tensor_lo[it.bucket], int32_t(it.tensor));
         P->bucket_tensor_hi[it.bucket] = std::max(P->bucket_tensor_hi[it.bucket], int32_t(it.tensor));
     }
+    int64_t data_items = 0, data_bytes = 0;
+    for (const rr_pack_item& it : P->pack_items)
+        if (it.kind <= RR_ITEM_BF16_SCALAR) {
+            ++data_items;
+            data_bytes += 2 * int64_t(it.row_len) * it.n_rows;
+        }
+    if (staged && data_bytes < RR_SHORT_ITEM * data_items)
+        pack_weight.overhead = RR_SHORT_ITEM_OVERHEAD;
     partition(P->pack_items, P->grid_blocks, P->pack_block_first, pack_weight);
     partition(P->unpack_items, P->unpack_grid_blocks, P->unpack_block_first, unpack_weight);
     bucket_units(P->unpack_items, P->unpack_bucket_first,
