@@ -216,7 +216,7 @@ rr_status rr_plan_create_ex(const rr_param* manifest, int32_t n_params,
                             const rr_src_layout* src, const rr_dst_layout* dst,
                             size_t bucket_bytes, const rr_plan_options* opts, rr_plan** out);
 
-/* Frees the plan's device tables, scratch and events.  Section 5.2.1 reserves
+/* Frees the plan's device tables and scratch.  Section 5.2.1 reserves
  * the transfer's memory ahead of the transfer so that it cannot run out of GPU
  * memory mid-sync; a plan is that reservation for the work tables, held from
  * creation until this call.  NULL is ignored.  No call of this plan may still
@@ -483,13 +483,12 @@ rr_status rr_plan_bucket_items(const rr_plan* plan, uint32_t* pack_first, uint32
  * kept in the call's scratch (the plan's for the blocking forms, the
  * caller's for rr_unpack_verify_async) or in a pooled slot; rr_unpack (either
  * engine) and rr_pack (bulk-copy engine) when they get one of the plan's 16
- * pooled slots.  A slot is free once the launch that last held it has
- * completed; when none is, a launch takes the slot handed out longest ago if
- * that slot's launch ran on the same stream, and the stream waits on the GPU
- * for that launch (which it would anyway).  A launch gets no slot when every
- * slot is held by another stream's launch still in flight, or when its stream
- * is capturing a graph; it then splits its items evenly over the grid, as the
- * register path's pack always does.  Which of these runs changes no output
+ * pooled slots, as the blocking verifies do.  A stream's launches use the
+ * slot that its last one held; another stream takes an idle one, whose last
+ * launch has ended.  A launch gets no slot when every slot is held by another
+ * stream's launch still in flight, or when its stream is capturing a graph; it
+ * then splits its items evenly over the grid, as the register path's pack
+ * always does.  Which of these runs changes no output
  * byte. */
 enum { RR_UNITS_PACK = 0, RR_UNITS_PACK_FULL = 1, RR_UNITS_UNPACK = 2 };
 rr_status rr_plan_work_units(const rr_plan* plan, int32_t which, int32_t* n_units,

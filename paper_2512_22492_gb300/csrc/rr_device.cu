@@ -80,6 +80,23 @@ struct ItemBounds {
     unsigned int* err;
 };
 
+// How a launch that compares checksums, or holds a pooled slot, ends.
+struct LaunchEnd {
+    unsigned long long* counters;  // {ticket, n_bad, max(ULLONG_MAX - bad index), claim}
+    // A verifying launch's answer, {n_bad, first_bad or -1} (NULL: none; the
+    // counters keep it, added up over a call's launches).  with_err: also
+    // result[2] = the plan's error word.
+    long long* result;
+    const unsigned int* err;
+    int32_t with_err;
+    // The launch holds a pooled slot: its last block leaves the slot (counters
+    // and sums) zeroed for the next launch, then stores `seq` at `done`, host
+    // memory, for a host thread that looks for a free slot.
+    int32_t slot;
+    unsigned long long* done;
+    unsigned long long seq;
+};
+
 // ---------------------------------------------------------------------------
 // Launch arguments (passed by value in the kernel parameter space, so that a
 // plan can run concurrently on several streams with different buffers).
@@ -110,9 +127,8 @@ struct UnpackArgs {
     const unsigned long long* weight_prefix;
     ItemBounds chk;
     // Verifying unpack only (as in VerifyArgs): per-bucket sums of the range
-    // [first_bucket, first_bucket + n_buckets), counters, expected sums, flags.
+    // [first_bucket, first_bucket + n_buckets), expected sums, flags.
     unsigned long long* sums;
-    unsigned long long* counters;
     const unsigned long long* expected;
     uint8_t* bad;
     int32_t first_bucket;
@@ -124,19 +140,19 @@ struct UnpackArgs {
     // Claimed work units (claim NULL: none, the split above).  unit_first holds
     // the first item of each of n_units units and one past the last; block g
     // walks unit g, then claims the next unclaimed unit (atomicAdd on *claim,
-    // zero at launch) until none are left.  claim is counters + 3.
+    // zero at launch) until none are left.  claim is end.counters + 3.
     const uint32_t* unit_first;
     unsigned long long* claim;
     uint32_t n_units;
-    uint32_t reset_claims;    // counters are a pooled slot's: its last block leaves them zero
-    long long* result;        // verifying: {n_bad, first_bad or -1} written at the end, or NULL
+    uint32_t pad_;
+    LaunchEnd end;
     const void* ptr[NPTR];    // (table mode) buckets bucket_lo, ..., then destination tensors
 };
 
 template <int NPTR>
 struct VerifyArgs {
     unsigned long long* sums;       // [n_buckets], zeroed
-    unsigned long long* counters;   // [4]: blocks done, n_bad, max(ULLONG_MAX - bad index)
+    LaunchEnd end;
     const unsigned long long* expected;   // indexed by global bucket
     uint8_t* bad;                   // optional [n_buckets]: 1 where the sum differs
     int32_t first_bucket;           // the range checked is [first_bucket, +n_buckets)
@@ -571,18 +587,9 @@ __global__ void __launch_bounds__(kThreads, RR_PACK_MIN_BLOCKS) rr_pack_kernel(c
 // no block waits for another).  sums[i] belongs to bucket first + i.
 // ---------------------------------------------------------------------------
 
-// The last block's result: counters[1] mismatches, the lowest one's index
-// from counters[2] (which holds ULLONG_MAX - index), or -1.
-__device__ __forceinline__ void write_result(unsigned long long* counters, long long* result) {
-    const unsigned long long nb = atomicAdd(&counters[1], 0ull);
-    result[0] = (long long)nb;
-    result[1] = nb ? (long long)(ULLONG_MAX - atomicAdd(&counters[2], 0ull)) : -1ll;
-}
-
-__device__ void compare_in_last_block(unsigned long long* counters,
-                                      const unsigned long long* sums,
-                                      const unsigned long long* expected, uint8_t* bad,
-                                      int32_t first, int32_t n, long long* result = nullptr) {
+// Whether this block is the last of its launch to get here (it then sees
+// everything that the others did before).
+__device__ __forceinline__ bool last_block_here(unsigned long long* counters) {
     __shared__ bool last;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -590,20 +597,50 @@ __device__ void compare_in_last_block(unsigned long long* counters,
         last = atomicAdd(&counters[0], 1ull) == gridDim.x - 1;
     }
     __syncthreads();
-    if (!last) return;
-    __threadfence();
+    if (last) __threadfence();
+    return last;
+}
+
+// Run by the whole last block: compares the sums of buckets first .. first + n
+// with the expected ones and writes the flags and the answer.
+__device__ __forceinline__ void compare_sums(const LaunchEnd& e, unsigned long long* sums,
+                                             const unsigned long long* expected, uint8_t* bad,
+                                             int32_t first, int32_t n) {
+    __shared__ unsigned long long n_bad, top;   // top: max(ULLONG_MAX - bad index)
+    if (threadIdx.x == 0) n_bad = top = 0;
+    __syncthreads();
     for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
         const int32_t b = first + i;
         const bool differs = __ldcg(sums + i) != expected[b];
         if (bad) bad[i] = differs ? 1 : 0;
         if (differs) {
-            atomicAdd(&counters[1], 1ull);
-            atomicMax(&counters[2], ULLONG_MAX - (unsigned long long)b);
+            atomicAdd(&n_bad, 1ull);
+            atomicMax(&top, ULLONG_MAX - (unsigned long long)b);
+        }
+        if (e.slot) sums[i] = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long nb = n_bad, tp = top;
+        if (!e.slot) {   // a call of several launches: what they found adds up
+            nb += atomicAdd(&e.counters[1], nb);
+            tp = max(tp, atomicMax(&e.counters[2], tp));
+        }
+        if (e.result) {
+            e.result[0] = (long long)nb;
+            e.result[1] = nb ? (long long)(ULLONG_MAX - tp) : -1ll;
+            if (e.with_err) e.result[2] = (long long)*(const volatile unsigned int*)e.err;
         }
     }
-    if (result) {
-        __syncthreads();
-        if (threadIdx.x == 0) write_result(counters, result);
+}
+
+// Run by the whole last block once it has read and zeroed the slot's sums.
+__device__ __forceinline__ void release_slot(const LaunchEnd& e) {
+    if (threadIdx.x < 4) e.counters[threadIdx.x] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence_system();
+        *(volatile unsigned long long*)e.done = e.seq;
     }
 }
 
@@ -701,25 +738,12 @@ __global__ void __launch_bounds__(RegUnpackShape<VERIFY>::kBlock, 4) rr_unpack_k
         i0 = a.unit_first[u];
         i1 = a.unit_first[u + 1];
     }
-    if (a.claim && a.reset_claims) {
-        // A pooled slot's counters go back to zero for its next launch: the
-        // block that takes the last ticket (counters[0]) resets them.  Every
-        // block gets here only after its last claim has returned.
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            if (atomicAdd(&a.counters[0], 1ull) == gridDim.x - 1) {
-                __threadfence();
-                atomicExch(a.claim, 0ull);
-                atomicExch(&a.counters[0], 0ull);
-            }
-        }
-    }
-    if (VERIFY) {
-        if (cur != 0xFFFFFFFFu) flush(a.sums + (cur - a.first_bucket), acc);
-        compare_in_last_block(a.counters, a.sums, a.expected, a.bad, a.first_bucket,
-                              a.n_buckets, a.result);
-    }
+    // Every block gets here only after its last claim has returned.
+    if (VERIFY && cur != 0xFFFFFFFFu) flush(a.sums + (cur - a.first_bucket), acc);
+    if (!VERIFY && !a.end.slot) return;
+    if (!last_block_here(a.end.counters)) return;
+    if (VERIFY) compare_sums(a.end, a.sums, a.expected, a.bad, a.first_bucket, a.n_buckets);
+    if (a.end.slot) release_slot(a.end);
 }
 
 // ---------------------------------------------------------------------------
@@ -759,7 +783,9 @@ __global__ void __launch_bounds__(kThreads, 4) rr_verify_kernel(const __grid_con
     }
     if (cur != 0xFFFFFFFFu) flush(a.sums + cur, acc);
 
-    compare_in_last_block(a.counters, a.sums, a.expected, a.bad, a.first_bucket, a.n_buckets);
+    if (!last_block_here(a.end.counters)) return;
+    compare_sums(a.end, a.sums, a.expected, a.bad, a.first_bucket, a.n_buckets);
+    if (a.end.slot) release_slot(a.end);
 }
 
 // ---------------------------------------------------------------------------
@@ -860,7 +886,7 @@ struct BulkArgs {
     int32_t bucket_lo;           // table mode: the first bucket the table holds
     int32_t pad_;
     unsigned long long* sums;    // pack: sums by global bucket; verify: range sums
-    unsigned long long* counters;// {ticket, n_bad, max(~0 - bad index), claim}
+    LaunchEnd end;
     const unsigned long long* expected;
     uint8_t* bad;
     int32_t first_bucket;        // the call's range [first_bucket, first_bucket + n_buckets)
@@ -869,19 +895,15 @@ struct BulkArgs {
     // Claimed work units (NULL: none).  block_first then holds the first item
     // of each of n_units units (and one past the last): unit g < gridDim.x is
     // block g's own, the rest go to whichever block asks next (atomicAdd on
-    // *claim = counters[3], zero at launch).
+    // *claim = end.counters[3], zero at launch).
     unsigned long long* claim;
     uint32_t n_units;
-    // The launch holds a pooled slot (counters, and sums for pack and the
-    // verifying unpack): its last block leaves them zero for the slot's next
-    // launch.
-    uint32_t reset_claims;
+    uint32_t pad2_;
     // Bytes of each source buffer, when some are not a multiple of 16 (else
     // NULL): a window of whole 16-byte words must not reach past a buffer's end.
     const int64_t* src_bytes;
     uint64_t bucket_bytes;
     unsigned long long* sums_out;  // pack through a slot: checksums[b] = sums[b] at the end
-    long long* result;             // verifying unpack: {n_bad, first_bad or -1}, or NULL
     const void* ptr[NPTR];
 };
 
@@ -1233,7 +1255,6 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
     __shared__ __align__(8) uint64_t full[kStages], empty[kStages];
     __shared__ Piece meta[kStages];
     __shared__ rr_pack_item fan_dst[MODE == 0 ? kStages : 1][kMaxFanDst];   // PC_FAN slices
-    __shared__ bool last_block;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr bool kSum = MODE != 1;
 
@@ -1796,43 +1817,19 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
     // finishes the launch: the verifying unpack compares the sums (and writes
     // the result); a pack through a slot writes its checksums out of the
     // slot's sums; a launch holding a slot leaves it zeroed.
-    if (MODE != 2 && !a.reset_claims) return;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last_block = atomicAdd(&a.counters[0], 1ull) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last_block) return;
-    __threadfence();
-    constexpr uint32_t kBT = BulkShape<MODE>::kThreads;
-    if constexpr (MODE == 2) {
-        for (int32_t i = threadIdx.x; i < a.n_buckets; i += kBT) {
-            const int32_t b = a.first_bucket + i;
-            const unsigned long long got = __ldcg(a.sums + i);
-            const bool differs = got != a.expected[b];
-            if (a.bad) a.bad[i] = differs ? 1 : 0;
-            if (differs) {
-                atomicAdd(&a.counters[1], 1ull);
-                atomicMax(&a.counters[2], ULLONG_MAX - (unsigned long long)b);
-            }
-            if (a.reset_claims) a.sums[i] = 0;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0 && a.result) write_result(a.counters, a.result);
-    }
+    if (MODE != 2 && !a.end.slot) return;
+    if (!last_block_here(a.end.counters)) return;
+    if constexpr (MODE == 2)
+        compare_sums(a.end, a.sums, a.expected, a.bad, a.first_bucket, a.n_buckets);
     if constexpr (MODE == 0) {
         if (a.sums_out)
-            for (int32_t i = threadIdx.x; i < a.n_buckets; i += kBT) {
+            for (int32_t i = threadIdx.x; i < a.n_buckets; i += BulkShape<MODE>::kThreads) {
                 const int32_t b = a.first_bucket + i;
                 a.sums_out[b] = __ldcg(a.sums + b);
                 a.sums[b] = 0;
             }
     }
-    if (a.reset_claims) {
-        __syncthreads();
-        if (threadIdx.x < 4) atomicExch(&a.counters[threadIdx.x], 0ull);
-    }
+    if (a.end.slot) release_slot(a.end);
 }
 
 // Self-test of the bounded wait: waits on a barrier phase that nothing
@@ -1894,48 +1891,59 @@ rr_status check_plan(const rr_plan* P) {
     return RR_OK;
 }
 
-// Whether a kernel of this library may touch memory at p: the current GPU's
-// device (or managed) memory, pinned host memory mapped for the device, or -- on a device
-// that reads pageable host memory (address translation over the CPU's page
-// tables, as on Grace) -- any host memory.  Pageable memory elsewhere would
-// fault the GPU, so it is refused.
-bool reachable(const void* p, bool pageable_ok) {
+// What a pointer's memory is to a kernel of this library on device `dev` (the
+// current one), from one attribute query.  `reach`: kernels may touch it: this
+// GPU's device (or managed) memory, pinned host memory mapped for the device,
+// or -- on a device that reads pageable host memory (address translation over
+// the CPU's page tables, as on Grace) -- any host memory.  Pageable memory
+// elsewhere would fault the GPU, so it is refused.  `device`: device memory,
+// which the bulk engine may read and write (host memory takes the register
+// path).
+struct Memory {
+    bool reach, device;
+};
+Memory memory_at(const void* p, int dev, bool pageable_ok) {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
-        return pageable_ok;
+        return {pageable_ok, false};
     }
-    if (at.type == cudaMemoryTypeDevice) {   // this GPU's own memory only
-        int dev = -1;
-        return cudaGetDevice(&dev) == cudaSuccess && at.device == dev;
-    }
-    if (at.type == cudaMemoryTypeManaged) return true;
-    if (at.type == cudaMemoryTypeHost) return at.devicePointer != nullptr;
-    return pageable_ok;
+    if (at.type == cudaMemoryTypeDevice) return {at.device == dev, true};
+    if (at.type == cudaMemoryTypeManaged) return {true, false};
+    if (at.type == cudaMemoryTypeHost) return {at.devicePointer != nullptr, false};
+    return {pageable_ok, false};
 }
 
 // Pointer arrays: every entry 16-byte aligned; the first and the last entry
 // reachable from the device (arrays are expected to be of one kind of memory).
-rr_status check_ptrs(bool pageable_ok, const void* const* ptrs, int32_t n, const char* what) {
+// *on_device: both are device memory (an empty array counts as such).
+rr_status check_ptrs(int dev, bool pageable_ok, const void* const* ptrs, int32_t n,
+                     const char* what, bool* on_device = nullptr) {
     if (n > 0 && !ptrs) return rr_fail(RR_EINVAL, "%s array is NULL", what);
     for (int32_t i = 0; i < n; ++i)
         if (!aligned16(ptrs[i]))
             return rr_fail(RR_EINVAL, "%s[%d] is NULL or not 16-byte aligned", what, i);
-    for (int32_t i : {0, n - 1})
-        if (n > 0 && !reachable(ptrs[i], pageable_ok))
+    bool device = true;
+    for (int32_t i = 0; i < n; i += std::max(1, n - 1)) {
+        const Memory m = memory_at(ptrs[i], dev, pageable_ok);
+        if (!m.reach)
             return rr_fail(RR_EINVAL,
                            "%s[%d] is memory this GPU cannot reach (pageable host memory, or "
                            "another GPU's); use this GPU's memory or pinned host memory",
                            what, i);
+        device = device && m.device;
+    }
+    if (on_device) *on_device = device;
     return RR_OK;
 }
 
 // One buffer a kernel reads or writes (checksums, per-bucket flags): 16-byte
 // aligned (when `aligned` is asked) and reachable from the device.
-rr_status check_buf(bool pageable_ok, const void* p, const char* what, bool aligned = true) {
+rr_status check_buf(int dev, bool pageable_ok, const void* p, const char* what,
+                    bool aligned = true) {
     if (!p || (aligned && !aligned16(p)))
         return rr_fail(RR_EINVAL, "%s NULL or not 16-byte aligned", what);
-    if (!reachable(p, pageable_ok))
+    if (!memory_at(p, dev, pageable_ok).reach)
         return rr_fail(RR_EINVAL,
                        "%s is memory this GPU cannot reach (pageable host memory, or another "
                        "GPU's); use this GPU's memory or pinned host memory", what);
@@ -1980,7 +1988,7 @@ ItemBounds bounds_of(const rr_plan* P) {
     return b;
 }
 
-int32_t take_claim_slot(rr_plan* M, cudaStream_t s);
+int32_t take_slot(rr_plan* M, cudaStream_t s, LaunchEnd* end);
 template <int MODE>
 void work_units(const rr_plan* P, const Range& R, const uint32_t** first, uint32_t* n);
 
@@ -2032,7 +2040,7 @@ rr_status launch_pack(const rr_plan* P, Range R, const void* const* src, void* c
 template <int NPTR>
 rr_status launch_unpack(const rr_plan* P, Range R, const void* const* buckets, void* const* dst,
                         const uint64_t* checksums, uint8_t* bad, bool table, uint64_t stride,
-                        cudaStream_t s, long long* result = nullptr) {
+                        cudaStream_t s, long long* result, bool with_err) {
     UnpackArgs<NPTR> a;
     std::memset(&a, 0, sizeof a);
     a.items = P->d_unpack_items;
@@ -2044,12 +2052,14 @@ rr_status launch_unpack(const rr_plan* P, Range R, const void* const* buckets, v
     if (checksums) {
         const SumSlot q = sum_slot(P, R, bad);
         a.sums = q.sums;
-        a.counters = q.counters;
+        a.end.counters = q.counters;
         a.expected = (const unsigned long long*)checksums;
         a.bad = q.bad;
         a.first_bucket = R.b0;
         a.n_buckets = R.b1 - R.b0;
-        a.result = result;
+        a.end.result = result;
+        a.end.err = P->d_error;
+        a.end.with_err = with_err;
     }
     int32_t k = 0;
     if (table) {
@@ -2068,14 +2078,12 @@ rr_status launch_unpack(const rr_plan* P, Range R, const void* const* buckets, v
     std::unique_lock<std::mutex> lock(M->claim_mutex, std::defer_lock);
     int32_t slot = -1;
     if (checksums) {
-        a.claim = a.counters + 3;
+        a.claim = a.end.counters + 3;
         work_units<1>(P, R, &a.unit_first, &a.n_units);
     } else {
         lock.lock();
-        if ((slot = take_claim_slot(M, s)) >= 0) {
-            a.counters = P->d_slots + size_t(slot) * P->slot_words() + P->n_buckets;
-            a.claim = a.counters + 3;
-            a.reset_claims = 1;
+        if ((slot = take_slot(M, s, &a.end)) >= 0) {
+            a.claim = a.end.counters + 3;
             work_units<1>(P, R, &a.unit_first, &a.n_units);
         }
     }
@@ -2089,26 +2097,42 @@ rr_status launch_unpack(const rr_plan* P, Range R, const void* const* buckets, v
     else
         rr_unpack_kernel<NPTR, false, false><<<P->reg_unpack_grid, kThreads, 0, s>>>(a);
     RR_CUDA(cudaGetLastError());
-    cudaError_t e;
-    if (slot >= 0 && (e = cudaEventRecord(P->claim_done[slot], s)) != cudaSuccess) {
-        M->claim_retired[slot] = 1;   // its launch's end is unknown: never hand it out again
-        return cuda_fail(e, "cudaEventRecord");
-    }
+    if (slot >= 0) M->slot_seq[slot] = a.end.seq;
     return RR_OK;
 }
 
 template <int NPTR>
 rr_status launch_verify(const rr_plan* P, Range R, const void* const* buckets,
                         const uint64_t* checksums, uint8_t* bad, bool table, uint64_t stride,
-                        cudaStream_t s) {
+                        cudaStream_t s, bool may_slot, long long* result) {
     VerifyArgs<NPTR> a;
     std::memset(&a, 0, sizeof a);
     const int32_t n = R.b1 - R.b0;
-    const SumSlot q = sum_slot(P, R, bad);
-    a.sums = q.sums;
-    a.counters = q.counters;
+    // One launch for the whole call sums into a pooled slot when one is free;
+    // otherwise the plan's scratch is zeroed first (here, or by the caller).
+    rr_plan* M = const_cast<rr_plan*>(P);   // the slot pool is mutable state
+    std::unique_lock<std::mutex> lock(M->claim_mutex, std::defer_lock);
+    int32_t slot = -1;
+    if (may_slot) {
+        lock.lock();
+        slot = take_slot(M, s, &a.end);
+    }
+    if (slot >= 0) {
+        a.sums = a.end.counters - P->n_buckets;
+        a.bad = bad;
+    } else {
+        if (may_slot)
+            RR_CUDA(cudaMemsetAsync(P->d_verify_scratch, 0,
+                                    (size_t(n) + 4) * sizeof(unsigned long long), s));
+        const SumSlot q = sum_slot(P, R, bad);
+        a.sums = q.sums;
+        a.end.counters = q.counters;
+        a.bad = q.bad;
+    }
+    a.end.result = result;
+    a.end.err = P->d_error;
+    a.end.with_err = 1;
     a.expected = (const unsigned long long*)checksums;
-    a.bad = q.bad;
     a.first_bucket = R.b0;
     a.bucket_bytes = (uint64_t)P->bucket_bytes;
     a.chunk_bytes = (uint64_t)std::min<int64_t>(kVerifyChunk, P->bucket_bytes);
@@ -2124,69 +2148,52 @@ rr_status launch_verify(const rr_plan* P, Range R, const void* const* buckets,
     }
     rr_verify_kernel<NPTR><<<P->verify_grid_blocks, kThreads, 0, s>>>(a);
     RR_CUDA(cudaGetLastError());
+    if (slot >= 0) M->slot_seq[slot] = a.end.seq;
     return RR_OK;
 }
 
-// The bulk engine reads and writes device memory only; buffers in host memory
-// (a snapshot to pinned host buckets) take the register path.  One call's
-// arrays are expected to be all device or all host memory: the first and
-// last pointer of each array are checked.
-bool device_resident(const void* p) {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice;
-}
-
-bool all_device(const void* const* ptrs, int32_t n) {
-    return n == 0 || (device_resident(ptrs[0]) && device_resident(ptrs[n - 1]));
-}
-
-// A pooled slot for a launch on `s`, or -1.  A slot whose last launch has
-// completed is free.  When none is, the slot handed out longest ago is taken
-// if its last launch ran on `s` itself: `s` then waits (on the GPU) for that
-// launch's event, which costs nothing since the stream runs its work in order
-// anyway.  Otherwise (every slot held by another stream's launch in flight, or
-// `s` capturing a graph -- a captured launch replays whenever the graph does)
-// there is none.  The caller holds claim_mutex and records claim_done[slot]
-// after the launch.  A slot is all zero when handed out: zeroed once at plan
-// creation, then by the last block of each launch that held it.
-int32_t take_claim_slot(rr_plan* M, cudaStream_t s) {
+// A pooled slot for a launch on `s`, or -1; fills in *end for it.  The slot that
+// the stream's own last launch held serves again: a stream runs its launches
+// in order, so that one is done with it first (a bulk kernel touches its slot
+// only past griddepcontrol.wait).  Otherwise a free one is taken, one whose
+// last launch has stored its number in the slot's word of host memory: no
+// event is recorded or queried (they cost about 1 us of host time each, and an
+// event between two kernels keeps the second from starting its prologue under
+// the first's tail).  None is left when every slot is held by another stream's
+// launch still in flight, or when `s` is capturing a graph (a captured launch
+// replays whenever the graph does).  The caller holds claim_mutex and sets
+// slot_seq[slot] = end->seq once the launch is enqueued (a launch that failed
+// leaves the slot as it was: zero, its last launch's number in place).  A slot
+// is all zero when handed out: zeroed once at plan creation, then by the last
+// block of each launch that held it.  Streams are told apart by their unique
+// id: a handle may come back for a new stream.
+int32_t take_slot(rr_plan* M, cudaStream_t s, LaunchEnd* end) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) {
+    unsigned long long id = 0;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess ||
+        (cs == cudaStreamCaptureStatusNone && cudaStreamGetId(s, &id) != cudaSuccess)) {
         cudaGetLastError();
         return -1;
     }
     if (cs != cudaStreamCaptureStatusNone) return -1;
-    // Querying an event is allowed to this thread even while another thread
-    // captures a graph.
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
+    auto idle = [&](int32_t k) {
+        return __atomic_load_n(M->h_slot_done + k * rr_plan::kDoneStride, __ATOMIC_ACQUIRE) ==
+               M->slot_seq[k];
+    };
     int32_t slot = -1;
+    for (int32_t k = 0; k < rr_plan::kClaimSlots && slot < 0; ++k)
+        if (M->slot_seq[k] != 0 && M->slot_stream[k] == id) slot = k;
     for (int32_t i = 0; i < rr_plan::kClaimSlots && slot < 0; ++i) {
         const int32_t k = (M->claim_next + i) % rr_plan::kClaimSlots;
-        if (M->claim_retired[k]) continue;
-        const cudaError_t q = cudaEventQuery(M->claim_done[k]);
-        if (q == cudaSuccess)
-            slot = k;
-        else if (q != cudaErrorNotReady)
-            cudaGetLastError();
+        if (idle(k)) slot = k;
     }
-    for (int32_t i = 0; i < rr_plan::kClaimSlots && slot < 0; ++i) {
-        const int32_t k = (M->claim_next + i) % rr_plan::kClaimSlots;
-        if (M->claim_retired[k] || M->claim_stream[k] != s) continue;
-        if (cudaStreamWaitEvent(s, M->claim_done[k], 0) == cudaSuccess)
-            slot = k;
-        else
-            cudaGetLastError();
-    }
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    if (slot >= 0) {
-        M->claim_next = (slot + 1) % rr_plan::kClaimSlots;
-        M->claim_stream[slot] = s;
-    }
+    if (slot < 0) return -1;
+    M->claim_next = (slot + 1) % rr_plan::kClaimSlots;
+    M->slot_stream[slot] = id;
+    end->counters = M->d_slots + size_t(slot) * M->slot_words() + M->n_buckets;
+    end->slot = 1;
+    end->done = M->h_slot_done + slot * rr_plan::kDoneStride;
+    end->seq = M->slot_seq[slot] + 1;
     return slot;
 }
 
@@ -2213,6 +2220,7 @@ struct BulkOpts {
     unsigned long long* zero = nullptr;   // without a slot, zero these words first (pack:
     size_t zero_words = 0;                //   the range's checksums; async verify: scratch)
     long long* result = nullptr;          // verifying unpack: write {n_bad, first_bad} here
+    bool result_err = false;              //   and the plan's error word after them
 };
 
 template <int NPTR, int MODE, bool CHECK, bool F16>
@@ -2295,13 +2303,11 @@ rr_status launch_bulk(const rr_plan* P, Range R, const void* const* src_shards,
     int32_t slot = -1;
     if (o.may_slot) {
         lock.lock();
-        slot = take_claim_slot(M, s);
+        slot = take_slot(M, s, &a.end);
     }
     if (slot >= 0) {
-        unsigned long long* area = P->d_slots + size_t(slot) * P->slot_words();
-        a.counters = area + P->n_buckets;
-        a.claim = a.counters + 3;
-        a.reset_claims = 1;
+        unsigned long long* area = a.end.counters - P->n_buckets;
+        a.claim = a.end.counters + 3;
         work_units<MODE>(P, R, &a.block_first, &a.n_units);
         if (MODE == 0 && o.zero) {          // the checksums come out of the slot's sums
             a.sums = area;
@@ -2316,7 +2322,7 @@ rr_status launch_bulk(const rr_plan* P, Range R, const void* const* src_shards,
         if (MODE == 2) {
             const SumSlot q = sum_slot(P, R, bad);
             a.sums = q.sums;
-            a.counters = q.counters;
+            a.end.counters = q.counters;
             a.claim = q.counters + 3;       // the call's work units, claimed through counters[3]
             a.bad = q.bad;
             work_units<MODE>(P, R, &a.block_first, &a.n_units);
@@ -2324,7 +2330,9 @@ rr_status launch_bulk(const rr_plan* P, Range R, const void* const* src_shards,
     }
     if (MODE == 2) {
         a.expected = (const unsigned long long*)checksums;
-        a.result = o.result;
+        a.end.result = o.result;
+        a.end.err = P->d_error;
+        a.end.with_err = o.result_err;
     }
     // The float16 instantiations exist for the pack only (F16 = MODE == 0 there).
     constexpr bool kF16 = MODE == 0;
@@ -2335,11 +2343,7 @@ rr_status launch_bulk(const rr_plan* P, Range R, const void* const* src_shards,
             : (P->check_items ? launch_bulk_kernel<NPTR, MODE, true, false>(grid, s, a)
                               : launch_bulk_kernel<NPTR, MODE, false, false>(grid, s, a));
     if (e != cudaSuccess) return cuda_fail(e, "bulk kernel launch");
-    cudaError_t er;
-    if (slot >= 0 && (er = cudaEventRecord(P->claim_done[slot], s)) != cudaSuccess) {
-        M->claim_retired[slot] = 1;   // its launch's end is unknown: never hand it out again
-        return cuda_fail(er, "cudaEventRecord");
-    }
+    if (slot >= 0) M->slot_seq[slot] = a.end.seq;
     return RR_OK;
 }
 
@@ -2372,10 +2376,15 @@ rr_status check_range(const rr_plan* P, int32_t first, int32_t n, Range* R) {
 rr_status pack_impl(const rr_plan* P, Range R, const void* const* src_shards, void* const* buckets,
                     uint64_t* checksums, cudaStream_t stream) {
     rr_status st;
-    if ((st = check_ptrs(P->pageable_ok != 0, src_shards, P->n_shards, "src_shards"))) return st;
-    if ((st = check_ptrs(P->pageable_ok != 0, (const void* const*)buckets, P->n_buckets, "buckets"))) return st;
+    bool src_device, buckets_device;
+    if ((st = check_ptrs(P->device, P->pageable_ok != 0, src_shards, P->n_shards, "src_shards",
+                         &src_device)))
+        return st;
+    if ((st = check_ptrs(P->device, P->pageable_ok != 0, (const void* const*)buckets, P->n_buckets,
+                         "buckets", &buckets_device)))
+        return st;
     if (R.b1 == R.b0) return RR_OK;
-    if ((st = check_buf(P->pageable_ok != 0, checksums, "checksums"))) return st;
+    if ((st = check_buf(P->device, P->pageable_ok != 0, checksums, "checksums"))) return st;
     uint64_t stride = 0;
     const bool table = !uniform((const void* const*)buckets, P->n_buckets, P->bucket_bytes, &stride);
     // Separately allocated buckets go through the pointer table after the
@@ -2387,9 +2396,7 @@ rr_status pack_impl(const rr_plan* P, Range R, const void* const* src_shards, vo
                        "%d source buffers leave no room for separately allocated buckets in one "
                        "launch's %d pointers; allocate the buckets as one equally spaced block",
                        P->n_shards, kLargePtrs);
-    const bool src_device = all_device(src_shards, P->n_shards);
-    const bool bulk = P->engine == RR_ENGINE_AUTO && src_device &&
-                      all_device((const void* const*)buckets, P->n_buckets);
+    const bool bulk = P->engine == RR_ENGINE_AUTO && src_device && buckets_device;
     const int32_t step = table ? cap : R.b1 - R.b0;
     const bool empty = P->pack_bucket_first[R.b0] == P->pack_bucket_first[R.b1];
     // One bulk launch writes the range's checksums itself (out of a pooled
@@ -2428,17 +2435,22 @@ rr_status pack_impl(const rr_plan* P, Range R, const void* const* src_shards, vo
     return RR_OK;
 }
 
-rr_status check_dst(const rr_plan* P, void* const* dst) {
-    if (P->n_tensors > 0 && !dst) return rr_fail(RR_EINVAL, "dst array is NULL");
-    for (int32_t t = 0; t < P->n_tensors; ++t)
+rr_status check_dst(const rr_plan* P, void* const* dst, bool* on_device) {
+    const int32_t n = P->n_tensors;
+    if (n > 0 && !dst) return rr_fail(RR_EINVAL, "dst array is NULL");
+    for (int32_t t = 0; t < n; ++t)
         if (P->tensor_numel[t] > 0 && !aligned16(dst[t]))
             return rr_fail(RR_EINVAL, "dst[%d] is NULL or not 16-byte aligned", t);
-    for (int32_t t : {0, P->n_tensors - 1})
-        if (P->n_tensors > 0 && P->tensor_numel[t] > 0 && !reachable(dst[t], P->pageable_ok != 0))
+    *on_device = true;
+    for (int32_t t = 0; t < n; t += std::max(1, n - 1)) {
+        const Memory m = memory_at(dst[t], P->device, P->pageable_ok != 0);
+        if (P->tensor_numel[t] > 0 && !m.reach)
             return rr_fail(RR_EINVAL,
                            "dst[%d] is memory this GPU cannot reach (pageable host memory, or "
                            "another GPU's); use this GPU's memory or pinned host memory",
                            t);
+        *on_device = *on_device && m.device;
+    }
     return RR_OK;
 }
 
@@ -2507,19 +2519,21 @@ rr_status launch_unpack_part(const rr_plan* P, const Range& S, bool bulk,
     Range Sr = S;
     Sr.full = S.full && P->engine == RR_ENGINE_REGISTERS;
     return small ? launch_unpack<kSmallPtrs>(P, Sr, buckets, dst, checksums, bad, sh.table,
-                                             sh.stride, stream, o.result)
+                                             sh.stride, stream, o.result, o.result_err)
                  : launch_unpack<kLargePtrs>(P, Sr, buckets, dst, checksums, bad, sh.table,
-                                             sh.stride, stream, o.result);
+                                             sh.stride, stream, o.result, o.result_err);
 }
 
 rr_status unpack_impl(const rr_plan* P, Range R, const void* const* buckets, void* const* dst,
                       cudaStream_t stream) {
     rr_status st;
-    if ((st = check_ptrs(P->pageable_ok != 0, buckets, P->n_buckets, "buckets"))) return st;
-    if ((st = check_dst(P, dst))) return st;
+    bool buckets_device, dst_device;
+    if ((st = check_ptrs(P->device, P->pageable_ok != 0, buckets, P->n_buckets, "buckets",
+                         &buckets_device)))
+        return st;
+    if ((st = check_dst(P, dst, &dst_device))) return st;
     if (P->unpack_bucket_first[R.b0] == P->unpack_bucket_first[R.b1]) return RR_OK;
-    const bool bulk = P->engine == RR_ENGINE_AUTO && all_device(buckets, P->n_buckets) &&
-                      all_device((const void* const*)dst, P->n_tensors);
+    const bool bulk = P->engine == RR_ENGINE_AUTO && buckets_device && dst_device;
     UnpackShape sh;
     if ((st = unpack_shape(P, R, buckets, &sh))) return st;
     for (const Range& S : sh.parts)
@@ -2530,16 +2544,18 @@ rr_status unpack_impl(const rr_plan* P, Range R, const void* const* buckets, voi
 
 rr_status read_error(const rr_plan* P, cudaStream_t stream);
 
-rr_status read_result(const rr_plan* P, int32_t n, int64_t* n_bad, int64_t* first_bad,
-                      cudaStream_t stream) {
-    RR_CUDA(cudaMemcpyAsync(P->h_verify_result, P->d_verify_scratch + n,
-                            4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream));
-    rr_status st = read_error(P, stream);
-    if (st) return st;
-    const unsigned long long nb = P->h_verify_result[1];
-    if (n_bad) *n_bad = (int64_t)nb;
-    if (first_bad) *first_bad = nb ? (int64_t)(ULLONG_MAX - P->h_verify_result[2]) : -1;
-    return nb ? RR_EMISMATCH : RR_OK;
+// The answer of a blocking verify: its last launch's last block writes it to
+// the plan's pinned words, with the plan's error word as it then is.
+rr_status read_result(const rr_plan* P, int64_t* n_bad, int64_t* first_bad, cudaStream_t stream) {
+    RR_CUDA(cudaStreamSynchronize(stream));
+    const long long* h = (const long long*)P->h_verify_result;
+    if (h[2]) {
+        rr_status st = read_error(P, stream);
+        if (st) return st;
+    }
+    if (n_bad) *n_bad = h[0];
+    if (first_bad) *first_bad = h[1];
+    return h[0] ? RR_EMISMATCH : RR_OK;
 }
 
 // Enqueues the verifying unpack of range R.  The stream-ordered form (R has
@@ -2552,19 +2568,19 @@ rr_status read_result(const rr_plan* P, int32_t n, int64_t* n_bad, int64_t* firs
 // first_bad} from the last launch's last block.
 rr_status enqueue_unpack_verify(const rr_plan* P, Range R, const void* const* buckets,
                                 const uint64_t* checksums, void* const* dst, uint8_t* bad,
-                                cudaStream_t stream, long long* result = nullptr) {
+                                bool on_device, cudaStream_t stream, long long* result) {
     const int32_t n = R.b1 - R.b0;
     unsigned long long* sc = R.scratch ? R.scratch : P->d_verify_scratch;
     UnpackShape sh;
     rr_status st = unpack_shape(P, R, buckets, &sh);
     if (st) return st;
-    const bool bulk = P->engine == RR_ENGINE_AUTO && all_device(buckets, P->n_buckets) &&
-                      all_device((const void* const*)dst, P->n_tensors);
-    if (bulk && R.scratch && sh.parts.size() == 1) {
+    const bool bulk = P->engine == RR_ENGINE_AUTO && on_device;
+    if (bulk && sh.parts.size() == 1) {
         BulkOpts o;
         o.zero = sc;
         o.zero_words = size_t(n) + 4;
         o.result = result;
+        o.result_err = !R.scratch;
         return launch_unpack_part(P, sh.parts[0], bulk, buckets, dst, checksums, bad, sh, stream,
                                   o);
     }
@@ -2577,6 +2593,7 @@ rr_status enqueue_unpack_verify(const rr_plan* P, Range R, const void* const* bu
         BulkOpts o;
         o.may_slot = false;
         o.result = i + 1 == sh.parts.size() ? result : nullptr;
+        o.result_err = !R.scratch;
         if ((st = launch_unpack_part(P, sh.parts[i], bulk, buckets, dst, checksums, bad, sh,
                                      stream, o)))
             return st;
@@ -2586,27 +2603,34 @@ rr_status enqueue_unpack_verify(const rr_plan* P, Range R, const void* const* bu
 
 rr_status check_unpack_verify_args(const rr_plan* P, Range R, const void* const* buckets,
                                    const uint64_t* checksums, void* const* dst,
-                                   const uint8_t* bad) {
+                                   const uint8_t* bad, bool* on_device) {
     rr_status st;
-    if ((st = check_ptrs(P->pageable_ok != 0, buckets, P->n_buckets, "buckets"))) return st;
-    if ((st = check_dst(P, dst))) return st;
-    if (R.b1 > R.b0 && (st = check_buf(P->pageable_ok != 0, checksums, "checksums"))) return st;
-    if (R.b1 > R.b0 && bad && (st = check_buf(P->pageable_ok != 0, bad, "bad", false))) return st;
+    bool buckets_device, dst_device;
+    if ((st = check_ptrs(P->device, P->pageable_ok != 0, buckets, P->n_buckets, "buckets",
+                         &buckets_device)))
+        return st;
+    if ((st = check_dst(P, dst, &dst_device))) return st;
+    *on_device = buckets_device && dst_device;
+    if (R.b1 > R.b0 && (st = check_buf(P->device, P->pageable_ok != 0, checksums, "checksums"))) return st;
+    if (R.b1 > R.b0 && bad && (st = check_buf(P->device, P->pageable_ok != 0, bad, "bad", false))) return st;
     return RR_OK;
 }
 
 rr_status unpack_verify_impl(const rr_plan* P, Range R, const void* const* buckets,
                              const uint64_t* checksums, void* const* dst, uint8_t* bad,
                              int64_t* n_bad, int64_t* first_bad, cudaStream_t stream) {
-    rr_status st = check_unpack_verify_args(P, R, buckets, checksums, dst, bad);
+    bool on_device;
+    rr_status st = check_unpack_verify_args(P, R, buckets, checksums, dst, bad, &on_device);
     if (st) return st;
     if (n_bad) *n_bad = 0;
     if (first_bad) *first_bad = -1;
     if (R.b1 == R.b0) return RR_OK;
     rr_plan* M = const_cast<rr_plan*>(P);   // the scratch area is the only mutable state
     std::lock_guard<std::mutex> lock(M->verify_mutex);
-    if ((st = enqueue_unpack_verify(P, R, buckets, checksums, dst, bad, stream))) return st;
-    return read_result(P, R.b1 - R.b0, n_bad, first_bad, stream);
+    if ((st = enqueue_unpack_verify(P, R, buckets, checksums, dst, bad, on_device, stream,
+                                    (long long*)P->h_verify_result)))
+        return st;
+    return read_result(P, n_bad, first_bad, stream);
 }
 
 // {n_bad, first_bad or -1} from a verifying pass's counters (NULL: an empty range).
@@ -2634,9 +2658,9 @@ rr_status verify_impl(const rr_plan* P, Range R, const void* const* buckets,
                       const uint64_t* checksums, uint8_t* bad, int64_t* n_bad, int64_t* first_bad,
                       cudaStream_t stream) {
     rr_status st;
-    if ((st = check_ptrs(P->pageable_ok != 0, buckets, P->n_buckets, "buckets"))) return st;
-    if (R.b1 > R.b0 && (st = check_buf(P->pageable_ok != 0, checksums, "checksums"))) return st;
-    if (R.b1 > R.b0 && bad && (st = check_buf(P->pageable_ok != 0, bad, "bad", false))) return st;
+    if ((st = check_ptrs(P->device, P->pageable_ok != 0, buckets, P->n_buckets, "buckets"))) return st;
+    if (R.b1 > R.b0 && (st = check_buf(P->device, P->pageable_ok != 0, checksums, "checksums"))) return st;
+    if (R.b1 > R.b0 && bad && (st = check_buf(P->device, P->pageable_ok != 0, bad, "bad", false))) return st;
     if (n_bad) *n_bad = 0;
     if (first_bad) *first_bad = -1;
     if (R.b1 == R.b0) return RR_OK;
@@ -2646,22 +2670,27 @@ rr_status verify_impl(const rr_plan* P, Range R, const void* const* buckets,
     rr_plan* M = const_cast<rr_plan*>(P);   // the scratch area is the only mutable state
     std::lock_guard<std::mutex> lock(M->verify_mutex);
     const int32_t n = R.b1 - R.b0;
-    RR_CUDA(cudaMemsetAsync(P->d_verify_scratch, 0, (size_t(n) + 4) * sizeof(unsigned long long),
-                            stream));
     // Separately allocated buckets: one launch per run of buckets that fits the
     // pointer table, sharing the call's counters (ticket reset in between).
     const int32_t step = table ? kLargePtrs : n;
+    const bool one = step >= n;
+    if (!one)
+        RR_CUDA(cudaMemsetAsync(P->d_verify_scratch, 0,
+                                (size_t(n) + 4) * sizeof(unsigned long long), stream));
     for (int32_t b = R.b0; b < R.b1; b += step) {
         const int32_t e = std::min(R.b1, b + step);
         if (b > R.b0)
             RR_CUDA(cudaMemsetAsync(P->d_verify_scratch + n, 0, sizeof(unsigned long long), stream));
         const Range S{b, e, false, nullptr, 0, -1, R.b0, n};
+        long long* result = e == R.b1 ? (long long*)P->h_verify_result : nullptr;
         st = (!table || e - b <= kSmallPtrs)
-                 ? launch_verify<kSmallPtrs>(P, S, buckets, checksums, bad, table, stride, stream)
-                 : launch_verify<kLargePtrs>(P, S, buckets, checksums, bad, table, stride, stream);
+                 ? launch_verify<kSmallPtrs>(P, S, buckets, checksums, bad, table, stride, stream,
+                                             one, result)
+                 : launch_verify<kLargePtrs>(P, S, buckets, checksums, bad, table, stride, stream,
+                                             one, result);
         if (st) return st;
     }
-    return read_result(P, n, n_bad, first_bad, stream);
+    return read_result(P, n_bad, first_bad, stream);
 }
 
 }  // namespace
@@ -2733,7 +2762,9 @@ rr_status rr_device_upload(rr_plan* P) {
                                            sizeof(unsigned long long))) != cudaSuccess ||
         (e = cudaMalloc((void**)&P->d_verify_scratch,
                         (size_t(P->n_buckets) + 4) * sizeof(unsigned long long))) != cudaSuccess ||
-        (e = cudaHostAlloc((void**)&P->h_verify_result, 5 * sizeof(unsigned long long),
+        (e = cudaHostAlloc((void**)&P->h_verify_result,
+                           (8 + rr_plan::kClaimSlots * rr_plan::kDoneStride) *
+                               sizeof(unsigned long long),
                            cudaHostAllocDefault)) != cudaSuccess ||
         (e = cudaMalloc((void**)&P->d_error, sizeof(unsigned int))) != cudaSuccess ||
         (e = cudaMemset(P->d_error, 0, sizeof(unsigned int))) != cudaSuccess ||
@@ -2753,8 +2784,9 @@ rr_status rr_device_upload(rr_plan* P) {
                   P->full_block_first.size() * sizeof(uint32_t))) != cudaSuccess)))
         return e == cudaErrorMemoryAllocation ? rr_fail(RR_ENOMEM, "device allocation failed")
                                               : cuda_fail(e, "plan upload");
-    for (cudaEvent_t& ev : P->claim_done)
-        RR_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    P->h_slot_done = P->h_verify_result + 8;
+    std::memset(P->h_verify_result, 0,
+                (8 + rr_plan::kClaimSlots * rr_plan::kDoneStride) * sizeof(unsigned long long));
     return RR_OK;
 }
 
@@ -2777,10 +2809,6 @@ void rr_device_release(rr_plan* P) {
     cudaFree(P->d_pack_unit_first);
     cudaFree(P->d_pack_whole_unit_first);
     cudaFree(P->d_slots);
-    for (cudaEvent_t& ev : P->claim_done) {
-        if (ev) cudaEventDestroy(ev);
-        ev = nullptr;
-    }
     cudaFree(P->d_verify_scratch);
     cudaFreeHost(P->h_verify_result);
     cudaFree(P->d_error);
@@ -2906,16 +2934,18 @@ extern "C" rr_status rr_unpack_verify_async(const rr_plan* P, int32_t first_buck
     Range R;
     rr_status st = check_plan(P);
     if (st || (st = check_range(P, first_bucket, n_buckets, &R))) return st;
-    if ((st = check_unpack_verify_args(P, R, buckets, checksums, dst, bad))) return st;
+    bool on_device;
+    if ((st = check_unpack_verify_args(P, R, buckets, checksums, dst, bad, &on_device))) return st;
     long long* res = result_address(result);
     if (!res)
         return rr_fail(RR_EINVAL, "result must be 8-byte aligned device or pinned host memory");
     if (R.b1 > R.b0) {
         if (!aligned16(scratch)) return rr_fail(RR_EINVAL, "scratch NULL or not 16-byte aligned");
-        if (!device_resident(scratch)) return rr_fail(RR_EINVAL, "scratch must be device memory");
+        if (!memory_at(scratch, P->device, false).device)
+            return rr_fail(RR_EINVAL, "scratch must be device memory");
         R.scratch = (unsigned long long*)scratch;
         // The launch's last block writes the result.
-        return enqueue_unpack_verify(P, R, buckets, checksums, dst, bad, stream, res);
+        return enqueue_unpack_verify(P, R, buckets, checksums, dst, bad, on_device, stream, res);
     }
     rr_verify_result_kernel<<<1, 1, 0, stream>>>(nullptr, res);   // an empty range
     RR_CUDA(cudaGetLastError());
@@ -2949,7 +2979,7 @@ extern "C" rr_status rr_clear_range(const rr_plan* P, int32_t first_bucket, int3
     Range R;
     rr_status st = check_plan(P);
     if (st || (st = check_range(P, first_bucket, n_buckets, &R))) return st;
-    if ((st = check_ptrs(P->pageable_ok != 0, (const void* const*)buckets, P->n_buckets, "buckets"))) return st;
+    if ((st = check_ptrs(P->device, P->pageable_ok != 0, (const void* const*)buckets, P->n_buckets, "buckets"))) return st;
     if (n_buckets == 0) return RR_OK;
     uint64_t stride = 0;
     if (uniform((const void* const*)buckets, P->n_buckets, P->bucket_bytes, &stride)) {
@@ -3027,7 +3057,7 @@ rr_status launch_static_verify(unsigned long long* scratch, int32_t grid, int32_
     VerifyArgs<NPTR> a;
     std::memset(&a, 0, sizeof a);
     a.sums = scratch;
-    a.counters = scratch + n_buckets;
+    a.end.counters = scratch + n_buckets;
     a.expected = (const unsigned long long*)checksums;
     a.bucket_bytes = bucket_bytes;
     a.chunk_bytes = std::min<uint64_t>((uint64_t)kVerifyChunk, bucket_bytes);
@@ -3062,9 +3092,9 @@ extern "C" rr_status rr_verify_noalloc(const void* const* buckets, int32_t n_buc
     int dev = 0, pageable = 0;
     RR_CUDA(cudaGetDevice(&dev));
     RR_CUDA(cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev));
-    rr_status st = check_ptrs(pageable != 0, buckets, n_buckets, "buckets");
+    rr_status st = check_ptrs(dev, pageable != 0, buckets, n_buckets, "buckets");
     if (st) return st;
-    if (n_buckets > 0 && (st = check_buf(pageable != 0, checksums, "checksums"))) return st;
+    if (n_buckets > 0 && (st = check_buf(dev, pageable != 0, checksums, "checksums"))) return st;
     if (n_bad) *n_bad = 0;
     if (first_bad) *first_bad = -1;
     if (n_buckets == 0) return RR_OK;

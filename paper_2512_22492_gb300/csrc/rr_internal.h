@@ -102,20 +102,23 @@ struct rr_plan {
     uint32_t* d_pack_unit_first = nullptr;
     uint32_t* d_pack_whole_unit_first = nullptr;
     // Pooled scratch of launches that need no per-call scratch: a slot is
-    // handed to a launch only once the event recorded after its previous
-    // launch has completed, and that launch's last block left it zeroed.  Slot
-    // k is slot_words() words at d_slots + k * slot_words(): per-bucket sums
-    // [n_buckets], then counters {ticket, n_bad, max(~0 - bad index), claim}.
+    // handed to the launch after its last one on the same stream, or to any
+    // once that launch has stored its number in the slot's word of pinned host
+    // memory, having left the slot zeroed.  Slot k is slot_words() words at
+    // d_slots + k * slot_words(): per-bucket sums [n_buckets], then counters
+    // {ticket, n_bad, max(~0 - bad index), claim}.
     static constexpr int kClaimSlots = 16;
+    static constexpr int kDoneStride = 8;          // words between the slots' host words
     unsigned long long* d_slots = nullptr;
     size_t slot_words() const { return size_t(n_buckets) + 4; }
-    cudaEvent_t claim_done[kClaimSlots] = {};
-    cudaStream_t claim_stream[kClaimSlots] = {};   // the stream of the slot's last launch
-    char claim_retired[kClaimSlots] = {};
+    unsigned long long* h_slot_done = nullptr;     // pinned: the number of the slot's last
+    unsigned long long slot_seq[kClaimSlots] = {}; //   launch that ended; of its last launch
+    unsigned long long slot_stream[kClaimSlots] = {};   // the id of that launch's stream
     int32_t claim_next = 0;
     std::mutex claim_mutex;
     unsigned long long* d_verify_scratch = nullptr;  // n_buckets sums + 4 counters
-    unsigned long long* h_verify_result = nullptr;   // pinned, 5 words (4 counters + error)
+    unsigned long long* h_verify_result = nullptr;   // pinned: {n_bad, first_bad, error word},
+                                                     //   [4] read_error's copy, then h_slot_done
     unsigned int* d_error = nullptr;                 // set by a kernel whose wait ran out
     std::mutex verify_mutex;
 };
