@@ -479,7 +479,8 @@ def _ptr_array(xs) -> ctypes.Array:
 def _stream(stream) -> int:
     if stream is None:
         import torch
-        return int(torch.cuda.current_stream().cuda_stream)
+        # The current stream's handle without a Stream object (3 us on Grace).
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return int(stream.cuda_stream)
