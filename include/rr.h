@@ -194,7 +194,8 @@ typedef struct {
     int32_t host_only;   /* 1: build the tables on the host only and touch no GPU; such
                             a plan can be queried and exported but not executed       */
     int32_t grid_blocks; /* persistent grid size; default: SMs x resident blocks      */
-    int64_t chunk_bytes; /* largest destination bytes per work item; default 64 KiB   */
+    int64_t chunk_bytes; /* largest destination bytes per work item; default 64 KiB,
+                            on small plans less (down to 8 KiB)                       */
     int32_t engine;      /* rr_engine                                                 */
     int32_t check_items; /* 1: every kernel checks each work item against the source,
                             bucket and tensor sizes of the plan before touching

@@ -90,8 +90,9 @@ struct LaunchEnd {
     const unsigned int* err;
     int32_t with_err;
     // The launch holds a pooled slot: its last block leaves the slot (counters
-    // and sums) zeroed for the next launch, then stores `seq` at `done`, host
-    // memory, for a host thread that looks for a free slot.
+    // and sums) zeroed for the next launch, then stores its number `seq` at
+    // `done` (device memory; the host copies these words when it runs short of
+    // slots).
     int32_t slot;
     unsigned long long* done;
     unsigned long long seq;
@@ -639,7 +640,7 @@ __device__ __forceinline__ void release_slot(const LaunchEnd& e) {
     if (threadIdx.x < 4) e.counters[threadIdx.x] = 0;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence_system();
+        __threadfence();
         *(volatile unsigned long long*)e.done = e.seq;
     }
 }
@@ -1243,8 +1244,14 @@ __device__ __forceinline__ char* bulk_bucket(const BulkArgs<NPTR>& a, uint32_t b
 
 // MODE 0: pack, 1: unpack, 2: unpack with checksum comparison.  CHECK: check
 // every item against the plan's buffers first (the check_items option).  F16
-// (pack only): the rollout's elements are float16, else bfloat16.
-template <int NPTR, int MODE, bool CHECK, bool F16>
+// (pack only): the rollout's elements are float16, else bfloat16.  FULL: the
+// table may hold elements of any alignment, fan-out heads or runs of short
+// items; the lean kernel (vector items and zero fills alone) has two fifths of
+// the code, and on launches of a few microseconds fetching code counts: a pack
+// and a verifying unpack of 1 K elements in turn take 10.5 us with the full
+// kernels on GB300 and 8.8 us with the lean ones, of 16 M elements 39.4 and
+// 34.2 us.
+template <int NPTR, int MODE, bool CHECK, bool F16, bool FULL>
 __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(const __grid_constant__ BulkArgs<NPTR> a) {
     static_assert(MODE == 0 || !F16, "the destination type matters to the pack only");
     using D = DstCast<F16>;
@@ -1254,7 +1261,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
     extern __shared__ __align__(128) char stage_mem[];
     __shared__ __align__(8) uint64_t full[kStages], empty[kStages];
     __shared__ Piece meta[kStages];
-    __shared__ rr_pack_item fan_dst[MODE == 0 ? kStages : 1][kMaxFanDst];   // PC_FAN slices
+    __shared__ rr_pack_item fan_dst[MODE == 0 && FULL ? kStages : 1][kMaxFanDst];   // PC_FAN slices
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr bool kSum = MODE != 1;
 
@@ -1283,8 +1290,9 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
     }
     // Everything else (sources, buckets, tensors, sums, counters) may be the
     // previous kernel's output: wait for it to complete.  A no-op when the
-    // launch did not overlap a previous kernel.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // launch did not overlap a previous kernel.  (The producer has its first
+    // items on the way by then.)
+    if (warp != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
@@ -1309,12 +1317,12 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
             if constexpr (MODE == 0) {
                 // A fan-out piece carries its destination items in shared memory
                 // (each lane's from registers: loaded once per head, not per piece).
-                if (p.kind == PC_FAN && lane < p.n) fan_dst[s][lane] = fan_mine;
+                if (FULL && p.kind == PC_FAN && lane < p.n) fan_dst[s][lane] = fan_mine;
             }
             const uint32_t stage = smem_u32(stage_mem + s * kStageBytes);
             const uint32_t row_bytes = p.row_len * p.es;
             if (how == kGather) gather_async(stage, fb, p.src, p.src_stride, p.rows, row_bytes, lane);
-            if (how == kRag) rag_async(stage, fb, p, lane);
+            if (FULL && how == kRag) rag_async(stage, fb, p, lane);
             __syncwarp();
             const bool rows_bulk = how == kBulk && p.rows > 1 && p.src_stride != row_bytes;
             if (lane == 0) {
@@ -1348,7 +1356,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
         unsigned long long pending = 0;
         bool claimed = false;
         auto next_range = [&](uint32_t* it) -> bool {
-            if (!a.claim) return false;
+            if (!a.claim || gridDim.x >= a.n_units) return false;   // every unit has its block
             if (!claimed && lane == 0) pending = atomicAdd(a.claim, 1ull);
             claimed = true;
             const unsigned long long u = gridDim.x + __shfl_sync(0xFFFFFFFFu, pending, 0);
@@ -1465,6 +1473,8 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
             ++count;
             return taken;
         };
+        if (i0 < i1) window_to(i0);
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         for (uint32_t it = i0; ok; ++it) {
             if (it >= i1) {
                 bool more = true;
@@ -1506,7 +1516,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                 off = d.dst_off;
                 p.es = (uint16_t)es;
                 p.sum_bucket = d.bucket;
-                if (d.kind == RR_ITEM_FAN_F32 || d.kind == RR_ITEM_FAN_BF16) {
+                if (FULL && (d.kind == RR_ITEM_FAN_F32 || d.kind == RR_ITEM_FAN_BF16)) {
                     // Whole rows of the slices' span, staged once; the destination
                     // items that follow the head are read by the consumers.
                     const uint32_t rb = L * es, nd = d.dst_off;
@@ -1545,7 +1555,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                     dst = bulk_bucket(a, d.bucket, a.n_shards) + d.dst_off;
                     if (d.kind == RR_ITEM_F32_VEC || d.kind == RR_ITEM_BF16_VEC) {
                         p.kind = es == 4 ? PC_CAST : PC_COPY;
-                        if (R == 1 && L * es <= (uint32_t)kStageBytes / 2) {
+                        if (FULL && R == 1 && L * es <= (uint32_t)kStageBytes / 2) {
                             const uint32_t taken = emit_joined(it, d, es, dst);
                             if (taken > 1 || !ok) {
                                 it += taken - 1;
@@ -1590,7 +1600,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
             }
             step = (uint32_t)kStageBytes / p.es;
             whole = R;
-            if (how == kRag) {
+            if (FULL && how == kRag) {
                 p.kind = PC_RAG;
                 k = (uint32_t)kStageBytes / rag_pitch(L, p.es);
                 step = ((uint32_t)kStageBytes - 16) / p.es & ~7u;
@@ -1616,9 +1626,9 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                         p.rows = min(k, whole - r);
                         p.row_len = L;
                     }
-                } else if (c < in) {
+                } else if (FULL && c < in) {
                     p.row_len = min(step, in - c);
-                } else {
+                } else if (FULL) {
                     p.rows = R - whole;
                     p.row_len = L - in;
                     p.kind = PC_SCALAR;
@@ -1628,7 +1638,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                 p.src = src + r * sstride + (uint64_t)c * p.es;
                 p.dst = dst ? dst + 2ull * ((uint64_t)r * L + c) : nullptr;
                 p.sum_off = off + 2u * (r * L + c);
-                if (MODE == 0 && fan) {
+                if (MODE == 0 && FULL && fan) {
                     p.n = fan;
                     p.sum_off = r;   // first row of this piece within the item
                 }
@@ -1714,6 +1724,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                 }
                 break;
             case PC_SCALAR:
+                if constexpr (FULL)
                 for (uint32_t e = ct; e < p.n; e += kCT) {
                     const uint32_t r = e / p.row_len, cc = e - r * p.row_len;
                     const char* q = p.src + r * p.src_stride + (uint64_t)cc * p.es;
@@ -1723,7 +1734,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                     if (kSum) acc += (unsigned long long)h << (8 * ((p.sum_off + 2 * e) & 7));
                 }
                 break;
-            case PC_RAG: {
+            case PC_RAG: if constexpr (FULL) {
                 unsigned long long am;
                 if (MODE == 0 && p.es == 4)
                     am = p.rows == 1 ? rag_run<D, 4>(st, p, ct, kCT)
@@ -1732,10 +1743,10 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                     am = MODE != 0 || p.rows == 1 ? rag_run<D, 2>(st, p, ct, kCT)
                                                   : rag_rows<D, 2>(st, p, ct, kCT);
                 if (kSum) acc += am;
-                break;
             }
+                break;
             case PC_FAN:   // pack only
-                if constexpr (MODE == 0) {
+                if constexpr (MODE == 0 && FULL) {
                     // Units of work: each slice's 16-byte output vectors in q parts
                     // (q spreads the slices over all consumer warps, whatever the
                     // number of rows staged); one warp per unit.  nd <= kMaxFanDst
@@ -1804,7 +1815,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
         if (lane == 0) mbar_arrive(smem_u32(&empty[s]));
     }
     if (kSum && cur != 0xFFFFFFFFu) flush(a.sums + (cur - sum_base), acc);
-    if constexpr (MODE == 0) {
+    if constexpr (MODE == 0 && FULL) {
 #pragma unroll
         for (uint32_t j = 0; j < kFanSlots; ++j)
             if (fan_bucket[j] != 0xFFFFFFFFu) flush(a.sums + fan_bucket[j], fan_acc[j]);
@@ -1844,9 +1855,9 @@ __global__ void rr_wait_selftest_kernel(unsigned int* err) {
     if (threadIdx.x == 0) mbar_wait(smem_u32(&bar), 0, err);
 }
 
-template <int NPTR, int MODE, bool CHECK = false, bool F16 = false>
+template <int NPTR, int MODE, bool CHECK = false, bool F16 = false, bool FULL = true>
 cudaError_t bulk_prepare() {
-    return cudaFuncSetAttribute(rr_bulk_kernel<NPTR, MODE, CHECK, F16>,
+    return cudaFuncSetAttribute(rr_bulk_kernel<NPTR, MODE, CHECK, F16, FULL>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 BulkShape<MODE>::kSmem);
 }
@@ -2155,13 +2166,16 @@ rr_status launch_verify(const rr_plan* P, Range R, const void* const* buckets,
 // A pooled slot for a launch on `s`, or -1; fills in *end for it.  The slot that
 // the stream's own last launch held serves again: a stream runs its launches
 // in order, so that one is done with it first (a bulk kernel touches its slot
-// only past griddepcontrol.wait).  Otherwise a free one is taken, one whose
-// last launch has stored its number in the slot's word of host memory: no
-// event is recorded or queried (they cost about 1 us of host time each, and an
-// event between two kernels keeps the second from starting its prologue under
-// the first's tail).  None is left when every slot is held by another stream's
-// launch still in flight, or when `s` is capturing a graph (a captured launch
-// replays whenever the graph does).  The caller holds claim_mutex and sets
+// only past griddepcontrol.wait).  Otherwise one that no launch has held yet,
+// or whose last launch is known to have ended: each launch leaves its number
+// in a device word, and a call that finds no slot has these words copied to
+// the host, on a stream of the plan's own, for the calls after it.  So a launch
+// costs its slot neither an event (about 1 us each to record and to query, and
+// one between two kernels keeps the second from starting its prologue under
+// the first's tail) nor a store to host memory (2 us at the end of a 10 us
+// kernel).  There is none when every slot is, as far as known, held by another
+// stream's launch, or when `s` is capturing a graph (a captured launch replays
+// whenever the graph does).  The caller holds claim_mutex and sets
 // slot_seq[slot] = end->seq once the launch is enqueued (a launch that failed
 // leaves the slot as it was: zero, its last launch's number in place).  A slot
 // is all zero when handed out: zeroed once at plan creation, then by the last
@@ -2176,23 +2190,30 @@ int32_t take_slot(rr_plan* M, cudaStream_t s, LaunchEnd* end) {
         return -1;
     }
     if (cs != cudaStreamCaptureStatusNone) return -1;
-    auto idle = [&](int32_t k) {
-        return __atomic_load_n(M->h_slot_done + k * rr_plan::kDoneStride, __ATOMIC_ACQUIRE) ==
-               M->slot_seq[k];
-    };
     int32_t slot = -1;
     for (int32_t k = 0; k < rr_plan::kClaimSlots && slot < 0; ++k)
         if (M->slot_seq[k] != 0 && M->slot_stream[k] == id) slot = k;
     for (int32_t i = 0; i < rr_plan::kClaimSlots && slot < 0; ++i) {
         const int32_t k = (M->claim_next + i) % rr_plan::kClaimSlots;
-        if (idle(k)) slot = k;
+        if (__atomic_load_n(M->h_slot_done + k, __ATOMIC_ACQUIRE) == M->slot_seq[k]) slot = k;
     }
-    if (slot < 0) return -1;
+    if (slot < 0) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // another thread may capture
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if ((!M->slot_copies &&
+             cudaStreamCreateWithFlags(&M->slot_copies, cudaStreamNonBlocking) != cudaSuccess) ||
+            cudaMemcpyAsync(M->h_slot_done, M->d_slot_done,
+                            rr_plan::kClaimSlots * sizeof(unsigned long long),
+                            cudaMemcpyDeviceToHost, M->slot_copies) != cudaSuccess)
+            cudaGetLastError();
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        return -1;
+    }
     M->claim_next = (slot + 1) % rr_plan::kClaimSlots;
     M->slot_stream[slot] = id;
     end->counters = M->d_slots + size_t(slot) * M->slot_words() + M->n_buckets;
     end->slot = 1;
-    end->done = M->h_slot_done + slot * rr_plan::kDoneStride;
+    end->done = M->d_slot_done + slot;
     end->seq = M->slot_seq[slot] + 1;
     return slot;
 }
@@ -2207,6 +2228,9 @@ void work_units(const rr_plan* P, const Range& R, const uint32_t** first, uint32
     if (MODE == 0 && R.full) {
         *first = P->d_pack_whole_unit_first;
         *n = uint32_t(P->pack_whole_unit_first.size() - 1);
+        if (*n == uint32_t(P->grid_blocks) + 1 &&   // no claimed unit that holds an item
+            P->pack_whole_unit_first[*n - 1] == P->pack_whole_unit_first[*n])
+            --*n;
     } else {
         const std::vector<uint32_t>& bu = MODE == 0 ? P->pack_bucket_unit : P->unpack_bucket_unit;
         *first = (MODE == 0 ? P->d_pack_unit_first : P->d_unpack_unit_first) + bu[R.b0];
@@ -2223,9 +2247,9 @@ struct BulkOpts {
     bool result_err = false;              //   and the plan's error word after them
 };
 
-template <int NPTR, int MODE, bool CHECK, bool F16>
+template <int NPTR, int MODE, bool CHECK, bool F16, bool FULL>
 cudaError_t launch_bulk_kernel(int32_t grid, cudaStream_t s, const BulkArgs<NPTR>& a) {
-    cudaError_t e = bulk_prepare<NPTR, MODE, CHECK, F16>();
+    cudaError_t e = bulk_prepare<NPTR, MODE, CHECK, F16, FULL>();
     if (e != cudaSuccess) return e;
     // Programmatic dependent launch: this grid's blocks may be scheduled while
     // the previous kernel on the stream drains (they wait for it to complete
@@ -2240,7 +2264,18 @@ cudaError_t launch_bulk_kernel(int32_t grid, cudaStream_t s, const BulkArgs<NPTR
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, rr_bulk_kernel<NPTR, MODE, CHECK, F16>, a);
+    return cudaLaunchKernelEx(&cfg, rr_bulk_kernel<NPTR, MODE, CHECK, F16, FULL>, a);
+}
+
+// The instantiation for a launch.  The checked kernels (a debugging aid) exist
+// with the large pointer table and the full code only.
+template <int NPTR, int MODE, bool F16>
+cudaError_t launch_bulk_kernel(bool check, bool full, int32_t grid, cudaStream_t s,
+                               const BulkArgs<NPTR>& a) {
+    if constexpr (NPTR == kLargePtrs)
+        if (check) return launch_bulk_kernel<NPTR, MODE, true, F16, true>(grid, s, a);
+    return full ? launch_bulk_kernel<NPTR, MODE, false, F16, true>(grid, s, a)
+                : launch_bulk_kernel<NPTR, MODE, false, F16, false>(grid, s, a);
 }
 
 template <int NPTR, int MODE>
@@ -2336,12 +2371,12 @@ rr_status launch_bulk(const rr_plan* P, Range R, const void* const* src_shards,
     }
     // The float16 instantiations exist for the pack only (F16 = MODE == 0 there).
     constexpr bool kF16 = MODE == 0;
-    const cudaError_t e =
-        MODE == 0 && P->dst_f16
-            ? (P->check_items ? launch_bulk_kernel<NPTR, MODE, true, kF16>(grid, s, a)
-                              : launch_bulk_kernel<NPTR, MODE, false, kF16>(grid, s, a))
-            : (P->check_items ? launch_bulk_kernel<NPTR, MODE, true, false>(grid, s, a)
-                              : launch_bulk_kernel<NPTR, MODE, false, false>(grid, s, a));
+    const bool check = P->check_items != 0;
+    const bool full = MODE == 0 ? (a.items == P->d_full_items || !P->pack_plain)
+                                : !P->unpack_plain;
+    const cudaError_t e = MODE == 0 && P->dst_f16
+                              ? launch_bulk_kernel<NPTR, MODE, kF16>(check, full, grid, s, a)
+                              : launch_bulk_kernel<NPTR, MODE, false>(check, full, grid, s, a);
     if (e != cudaSuccess) return cuda_fail(e, "bulk kernel launch");
     if (slot >= 0) M->slot_seq[slot] = a.end.seq;
     return RR_OK;
@@ -2417,7 +2452,7 @@ rr_status pack_impl(const rr_plan* P, Range R, const void* const* src_shards, vo
         const int32_t need = P->n_shards + (table ? e - b : 0);
         if (P->pack_bucket_first[b] == P->pack_bucket_first[e]) continue;
         if (bulk)
-            st = need <= kSmallPtrs
+            st = need <= kSmallPtrs && !P->check_items
                      ? launch_bulk<kSmallPtrs, 0>(P, S, src_shards, (const void* const*)buckets,
                                                   nullptr, checksums, nullptr, table, stride, stream,
                                                   o)
@@ -2502,8 +2537,9 @@ rr_status launch_unpack_part(const rr_plan* P, const Range& S, bool bulk,
                              const void* const* buckets, void* const* dst,
                              const uint64_t* checksums, uint8_t* bad, const UnpackShape& sh,
                              cudaStream_t stream, const BulkOpts& o = BulkOpts()) {
-    const bool small = (S.t_hi - S.t_lo + 1) + (sh.table ? S.b1 - S.b0 : 0) <= kSmallPtrs;
+    const bool few = (S.t_hi - S.t_lo + 1) + (sh.table ? S.b1 - S.b0 : 0) <= kSmallPtrs;
     if (bulk) {
+        const bool small = few && !P->check_items;
         if (checksums)
             return small ? launch_bulk<kSmallPtrs, 2>(P, S, nullptr, buckets, dst, checksums, bad,
                                                       sh.table, sh.stride, stream, o)
@@ -2518,7 +2554,7 @@ rr_status launch_unpack_part(const rr_plan* P, const Range& S, bool bulk,
     // the register grid.
     Range Sr = S;
     Sr.full = S.full && P->engine == RR_ENGINE_REGISTERS;
-    return small ? launch_unpack<kSmallPtrs>(P, Sr, buckets, dst, checksums, bad, sh.table,
+    return few ? launch_unpack<kSmallPtrs>(P, Sr, buckets, dst, checksums, bad, sh.table,
                                              sh.stride, stream, o.result, o.result_err)
                  : launch_unpack<kLargePtrs>(P, Sr, buckets, dst, checksums, bad, sh.table,
                                              sh.stride, stream, o.result, o.result_err);
@@ -2711,10 +2747,10 @@ rr_status rr_device_default_grid(rr_grids* g) {
     int bp = 0;
     RR_CUDA((bulk_prepare<kLargePtrs, 0>()));
     RR_CUDA((bulk_prepare<kLargePtrs, 2>()));
-    RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bp, rr_bulk_kernel<kLargePtrs, 0, false, false>,
+    RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bp, rr_bulk_kernel<kLargePtrs, 0, false, false, true>,
                                                           BulkShape<0>::kThreads,
                                                           BulkShape<0>::kSmem));
-    RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, rr_bulk_kernel<kLargePtrs, 2, false, false>,
+    RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, rr_bulk_kernel<kLargePtrs, 2, false, false, true>,
                                                           BulkShape<2>::kThreads,
                                                           BulkShape<2>::kSmem));
     g->reg_pack = sms * (p > 0 ? p : 1);
@@ -2756,15 +2792,15 @@ rr_status rr_device_upload(rr_plan* P) {
                 P->pack_unit_first.size() * sizeof(uint32_t))) != cudaSuccess ||
         (e = up((void**)&P->d_pack_whole_unit_first, P->pack_whole_unit_first.data(),
                 P->pack_whole_unit_first.size() * sizeof(uint32_t))) != cudaSuccess ||
-        (e = cudaMalloc((void**)&P->d_slots, rr_plan::kClaimSlots * P->slot_words() *
+        (e = cudaMalloc((void**)&P->d_slots, rr_plan::kClaimSlots * (P->slot_words() + 1) *
                                                  sizeof(unsigned long long))) != cudaSuccess ||
-        (e = cudaMemset(P->d_slots, 0, rr_plan::kClaimSlots * P->slot_words() *
+        (e = cudaMemset(P->d_slots, 0, rr_plan::kClaimSlots * (P->slot_words() + 1) *
                                            sizeof(unsigned long long))) != cudaSuccess ||
+
         (e = cudaMalloc((void**)&P->d_verify_scratch,
                         (size_t(P->n_buckets) + 4) * sizeof(unsigned long long))) != cudaSuccess ||
         (e = cudaHostAlloc((void**)&P->h_verify_result,
-                           (8 + rr_plan::kClaimSlots * rr_plan::kDoneStride) *
-                               sizeof(unsigned long long),
+                           (8 + rr_plan::kClaimSlots) * sizeof(unsigned long long),
                            cudaHostAllocDefault)) != cudaSuccess ||
         (e = cudaMalloc((void**)&P->d_error, sizeof(unsigned int))) != cudaSuccess ||
         (e = cudaMemset(P->d_error, 0, sizeof(unsigned int))) != cudaSuccess ||
@@ -2784,9 +2820,10 @@ rr_status rr_device_upload(rr_plan* P) {
                   P->full_block_first.size() * sizeof(uint32_t))) != cudaSuccess)))
         return e == cudaErrorMemoryAllocation ? rr_fail(RR_ENOMEM, "device allocation failed")
                                               : cuda_fail(e, "plan upload");
+    P->d_slot_done = P->d_slots + rr_plan::kClaimSlots * P->slot_words();
     P->h_slot_done = P->h_verify_result + 8;
     std::memset(P->h_verify_result, 0,
-                (8 + rr_plan::kClaimSlots * rr_plan::kDoneStride) * sizeof(unsigned long long));
+                (8 + rr_plan::kClaimSlots) * sizeof(unsigned long long));
     return RR_OK;
 }
 
@@ -2808,6 +2845,11 @@ void rr_device_release(rr_plan* P) {
     cudaFree(P->d_unpack_unit_first);
     cudaFree(P->d_pack_unit_first);
     cudaFree(P->d_pack_whole_unit_first);
+    if (P->slot_copies) {   // a copy of the done words may still be under way
+        cudaStreamSynchronize(P->slot_copies);
+        cudaStreamDestroy(P->slot_copies);
+    }
+    P->slot_copies = nullptr;
     cudaFree(P->d_slots);
     cudaFree(P->d_verify_scratch);
     cudaFreeHost(P->h_verify_result);

@@ -77,6 +77,8 @@ struct rr_plan {
     std::vector<rr_pack_item> full_items;       // whole-sync table with fan-out groups;
                                                 // empty when it would equal pack_items
     std::vector<uint32_t> full_block_first;     // grid_blocks + 1
+    bool pack_plain = false;          // pack_items / unpack_items hold vector items and zero
+    bool unpack_plain = false;        //   fills alone, no runs of short ones (the lean kernels)
     std::vector<uint32_t> unpack_bucket_first;  // n_buckets + 1: first unpack item of bucket b
     std::vector<int32_t> bucket_tensor_lo;      // n_buckets: lowest / highest destination
     std::vector<int32_t> bucket_tensor_hi;      //   tensor a bucket's unpack items write
@@ -103,17 +105,17 @@ struct rr_plan {
     uint32_t* d_pack_whole_unit_first = nullptr;
     // Pooled scratch of launches that need no per-call scratch: a slot is
     // handed to the launch after its last one on the same stream, or to any
-    // once that launch has stored its number in the slot's word of pinned host
-    // memory, having left the slot zeroed.  Slot k is slot_words() words at
-    // d_slots + k * slot_words(): per-bucket sums [n_buckets], then counters
-    // {ticket, n_bad, max(~0 - bad index), claim}.
+    // once that launch is known to have ended (it left the slot zeroed).  Slot
+    // k is slot_words() words at d_slots + k * slot_words(): per-bucket sums
+    // [n_buckets], then counters {ticket, n_bad, max(~0 - bad index), claim}.
     static constexpr int kClaimSlots = 16;
-    static constexpr int kDoneStride = 8;          // words between the slots' host words
     unsigned long long* d_slots = nullptr;
     size_t slot_words() const { return size_t(n_buckets) + 4; }
-    unsigned long long* h_slot_done = nullptr;     // pinned: the number of the slot's last
-    unsigned long long slot_seq[kClaimSlots] = {}; //   launch that ended; of its last launch
-    unsigned long long slot_stream[kClaimSlots] = {};   // the id of that launch's stream
+    unsigned long long slot_seq[kClaimSlots] = {};     // the slot's launches so far
+    unsigned long long slot_stream[kClaimSlots] = {};  // the id of the last one's stream
+    unsigned long long* d_slot_done = nullptr;         // the number of the last that ended,
+    unsigned long long* h_slot_done = nullptr;         //   and a pinned copy of some time ago,
+    cudaStream_t slot_copies = nullptr;                //   made on this stream
     int32_t claim_next = 0;
     std::mutex claim_mutex;
     unsigned long long* d_verify_scratch = nullptr;  // n_buckets sums + 4 counters

@@ -33,13 +33,19 @@ namespace {
 thread_local std::string g_error;
 
 constexpr int64_t kDefaultChunkBytes = 64 * 1024;
+#ifndef RR_MIN_CHUNK
+#define RR_MIN_CHUNK (8 * 1024)
+#endif
+constexpr int64_t kMinChunkBytes = RR_MIN_CHUNK;   // plans with less than an item per block:
+constexpr int64_t kItemsPerBlock = 4;              //   halved down to this until it has four
 // Balancing weights (build-time overridable for tuning sweeps).  Beyond its
 // bytes an item costs its copies' issue, by one producer warp.  Where short
-// items make up the table (a relay's pieces of 1 to 3 KiB, RR_SHORT_ITEM bytes
-// each on average at most) that is about 3 KiB of traffic an item: such a
-// relay's pack ran at 430, 371, 338, 287, 273 and 273 us with 0, 0.5, 1, 2, 3
-// and 4 KiB.  Tables of large items with a few short ones among them run the
-// same with each, and the odd-sized one best with 1 (244 us, 250 with 3).
+// items make up the table (a relay's pieces of 1 to 3 KiB; on average under
+// RR_SHORT_ITEM bytes and a quarter of the plan's largest) that is about 3 KiB
+// of traffic an item: such a relay's pack ran at 430, 371, 338, 287, 273 and 273
+// us with 0, 0.5, 1, 2, 3 and 4 KiB.  Tables of large items with a few short
+// ones among them run the same with each, and the odd-sized one best with 1
+// (244 us, 250 with 3).
 #ifndef RR_ITEM_OVERHEAD
 #define RR_ITEM_OVERHEAD 1024
 #endif
@@ -81,6 +87,11 @@ constexpr int64_t kMaxShardOffset = (int64_t(1) << 48) - 1;
 constexpr int64_t kMaxFanDst = 16;
 constexpr int64_t kFanMaxRowBytes = 48 * 1024;
 
+int64_t stream_bytes(const rr_plan* P) {
+    int64_t n = 0;
+    for (int64_t b : P->rank_stream_bytes) n += b;
+    return n;
+}
 int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 bool is_pow2(int64_t x) { return x > 0 && (x & (x - 1)) == 0; }
 
@@ -441,6 +452,17 @@ void partition(const std::vector<Item>& items, int32_t grid, std::vector<uint32_
     }
 }
 
+// A table that gives each block less than this is a launch of a few
+// microseconds, which every claim (a round trip to L2) would only lengthen: its
+// blocks get all of their work up front.  Measured on GB300: the pack of 8 M
+// elements (330 KiB a block) 14.8 us with claims, 11.7 without, of 16 M 20.6 and
+// 20.1; the verifying unpack (two blocks per SM) of 8 M (110 KiB a block) the
+// same, of 64 M (880 KiB) 45.0 and 45.8.
+constexpr int64_t kSmallPackShare = 1024 * 1024, kSmallUnitShare = 256 * 1024;
+bool small_table(int64_t total, int32_t grid, int64_t share) {
+    return total < share * std::max(1, grid);
+}
+
 // Claimed units get smaller toward the end of the table (guided
 // self-scheduling): a unit that starts with `rem` weight left before the end is
 // about rem / (2 * grid), clamped to [floor, unit_weight].  Blocks drain HBM at
@@ -503,7 +525,7 @@ void whole_units(const std::vector<Item>& items, int32_t grid, int64_t unit_weig
                  std::vector<uint32_t>& first, W w) {
     int64_t total = 0;
     for (const Item& it : items) total += w(it);
-    const int64_t own = total * kOwnShareNum / kOwnShareDen;
+    const int64_t own = small_table(total, grid, kSmallPackShare) ? total : total * kOwnShareNum / kOwnShareDen;
     first.assign(size_t(grid) + 1, uint32_t(items.size()));
     first[0] = 0;
     int64_t cum = 0;
@@ -529,13 +551,16 @@ void whole_units(const std::vector<Item>& items, int32_t grid, int64_t unit_weig
     if (first.size() == size_t(grid) + 1) first.push_back(uint32_t(items.size()));
 }
 
-// Claimed-unit weight for a table: about kUnitsPerBlock units per block of the
+// Claimed-unit weight for a table: one unit per block on a small plan (with
+// some room for the units that a bucket's end cuts short); else about kUnitsPerBlock units per block of the
 // grid, none above kUnitWeight (small enough to even out the finish), none
 // below kUnitWeight / 8 (each costs the producer one claim).
 template <class Item, class W>
 int64_t unit_weight_for(const std::vector<Item>& items, int32_t grid, W w) {
     int64_t total = 0;
     for (const Item& it : items) total += w(it);
+    if (small_table(total, grid, kSmallUnitShare))
+        return std::max<int64_t>(8 * 1024, total * 115 / 100 / std::max(1, grid));
     const int64_t per_block = total / (int64_t(kUnitsPerBlock) * std::max(1, grid));
     return std::min(kUnitWeight, std::max(kUnitWeight / 8, per_block));
 }
@@ -857,8 +882,16 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
             ++data_items;
             data_bytes += 2 * int64_t(it.row_len) * it.n_rows;
         }
-    if (staged && data_bytes < RR_SHORT_ITEM * data_items)
-        pack_weight.overhead = RR_SHORT_ITEM_OVERHEAD;
+    const bool short_items =
+        data_bytes < std::min<int64_t>(RR_SHORT_ITEM, P->chunk_bytes / 4) * data_items;
+    if (staged && short_items) pack_weight.overhead = RR_SHORT_ITEM_OVERHEAD;
+    P->pack_plain = !short_items;
+    for (const rr_pack_item& it : P->pack_items)
+        if (it.kind == RR_ITEM_F32_SCALAR || it.kind == RR_ITEM_BF16_SCALAR) P->pack_plain = false;
+    P->unpack_plain = true;
+    for (const rr_unpack_item& it : P->unpack_items)
+        if (it.kind == RR_ITEM_COPY_SCALAR || it.kind == RR_ITEM_READ_SCALAR)
+            P->unpack_plain = false;
     partition(P->pack_items, P->grid_blocks, P->pack_block_first, pack_weight);
     partition(P->unpack_items, P->unpack_grid_blocks, P->unpack_block_first, unpack_weight);
     bucket_units(P->unpack_items, P->unpack_bucket_first,
@@ -1004,6 +1037,16 @@ rr_status rr_plan_create_ex(const rr_param* manifest, int32_t n_params,
             if (opts && opts->grid_blocks > 0)
                 P->grid_blocks = P->unpack_grid_blocks = P->verify_grid_blocks = P->reg_pack_grid =
                     P->reg_unpack_grid = P->reg_vunpack_grid = opts->grid_blocks;
+            // Small plans (not an item for every block): smaller items, so that
+            // every block gets a few.  Pack and verifying unpack of 1, 2 and 4 M
+            // elements in turn on GB300: 15.5, 15.9 and 16.9 us with 64 KiB
+            // items, 12.6, 13.8 and 15.5 us with these; of 8 M, where every block
+            // has a 64 KiB item, 20.9 us, and 21.5 with smaller ones.
+            if (!(opts && opts->chunk_bytes) &&
+                stream_bytes(P) < P->chunk_bytes * P->grid_blocks)
+                while (P->chunk_bytes > kMinChunkBytes &&
+                       stream_bytes(P) < kItemsPerBlock * P->chunk_bytes * P->grid_blocks)
+                    P->chunk_bytes /= 2;
         }
         if (st == RR_OK) {
             build_tables(P, dst);
