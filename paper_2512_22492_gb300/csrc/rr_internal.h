@@ -2,6 +2,7 @@
 // the device code (rr_device.cu).  Not part of the public ABI.
 #pragma once
 
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -57,7 +58,8 @@ struct rr_plan {
     int32_t reg_vunpack_grid = 0;     // the register path's verifying unpack (its own block size)
     int32_t engine = RR_ENGINE_AUTO;
     int32_t dst_f16 = 0;              // the rollout's elements are float16 (else bfloat16)
-    int64_t chunk_bytes = 0;
+    int64_t chunk_bytes = 0;          // largest destination bytes of a pack item,
+    int64_t unpack_chunk_bytes = 0;   //   of an unpack item
     bool host_only = false;
     std::vector<rr_pack_item> pack_items;
     std::vector<uint32_t> pack_block_first;     // grid_blocks + 1
@@ -118,6 +120,7 @@ struct rr_plan {
     cudaStream_t slot_copies = nullptr;                //   made on this stream
     int32_t claim_next = 0;
     std::mutex claim_mutex;
+    std::atomic<uint64_t> prepared{0};   // bulk kernels whose shared memory is set up
     unsigned long long* d_verify_scratch = nullptr;  // n_buckets sums + 4 counters
     unsigned long long* h_verify_result = nullptr;   // pinned: {n_bad, first_bad, error word},
                                                      //   [4] read_error's copy, then h_slot_done

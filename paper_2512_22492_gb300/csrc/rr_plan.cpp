@@ -33,11 +33,8 @@ namespace {
 thread_local std::string g_error;
 
 constexpr int64_t kDefaultChunkBytes = 64 * 1024;
-#ifndef RR_MIN_CHUNK
-#define RR_MIN_CHUNK (8 * 1024)
-#endif
-constexpr int64_t kMinChunkBytes = RR_MIN_CHUNK;   // plans with less than an item per block:
-constexpr int64_t kItemsPerBlock = 4;              //   halved down to this until it has four
+constexpr int64_t kMinChunkBytes = 4 * 1024;   // smallest items of a small plan
+constexpr int64_t kSmallPlanItems = 2;         // items per block of a small plan
 // Balancing weights (build-time overridable for tuning sweeps).  Beyond its
 // bytes an item costs its copies' issue, by one producer warp.  Where short
 // items make up the table (a relay's pieces of 1 to 3 KiB; on average under
@@ -87,13 +84,25 @@ constexpr int64_t kMaxShardOffset = (int64_t(1) << 48) - 1;
 constexpr int64_t kMaxFanDst = 16;
 constexpr int64_t kFanMaxRowBytes = 48 * 1024;
 
-int64_t stream_bytes(const rr_plan* P) {
-    int64_t n = 0;
-    for (int64_t b : P->rank_stream_bytes) n += b;
-    return n;
-}
 int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 bool is_pow2(int64_t x) { return x > 0 && (x & (x - 1)) == 0; }
+
+// The item size of a plan on a grid: the plan's, or on a small plan (not such an
+// item for every block) a share of the stream that gives every block two.  A
+// block's ring has three stages, so that up to three items are under way at
+// once: with more, the last ones wait a round trip to memory (packing the
+// two-layer test model took 9.7 us with two 14 KiB items a block on GB300, 10.9
+// with three to four of 8 KiB, 14.1 with six to seven of 4 KiB, and 12.2 with
+// 64 KiB items for every other block; pack and verifying unpack of 1, 2 and 4 M
+// elements in turn 11.0, 11.9 and 14.7 us, with 64 KiB items 15.6, 16.1 and
+// 16.9).
+int64_t small_chunk(const rr_plan* P, int32_t grid) {
+    int64_t total = 0;
+    for (int64_t b : P->rank_stream_bytes) total += b;
+    if (total >= P->chunk_bytes * std::max(1, grid)) return P->chunk_bytes;
+    const int64_t share = align_up(total / (kSmallPlanItems * std::max(1, grid)) + 1, 1024);
+    return std::min(P->chunk_bytes, std::max(kMinChunkBytes, share));
+}
 
 // One member of a fan-out group: a column slice of the group's rows that lands
 // contiguously in rank `rank`'s stream at byte `pos`.
@@ -200,7 +209,7 @@ public:
             const int64_t pos = P->tensor_off[t] + x;
             const int64_t bl = pos / B, boff = pos - bl * B;
             // Pieces end on 16-byte boundaries of the tensor (as in pack_run).
-            int64_t len = std::min({nbytes - x, B - boff, P->chunk_bytes - x % 16});
+            int64_t len = std::min({nbytes - x, B - boff, P->unpack_chunk_bytes - x % 16});
             copy_piece(fb + bl, boff, t, x, len);
             x += len;
         }
@@ -214,7 +223,7 @@ public:
         while (a < b) {
             const int64_t bl = a / B;
             int64_t boff = a - bl * B;
-            int64_t len = std::min({b - a, B - boff, P->chunk_bytes});
+            int64_t len = std::min({b - a, B - boff, P->unpack_chunk_bytes});
             int64_t h = std::min((16 - boff % 16) % 16, len);
             if (h) {
                 emit_copy(RR_ITEM_READ_SCALAR, fb + bl, boff, -1, 0, h);
@@ -1037,16 +1046,11 @@ rr_status rr_plan_create_ex(const rr_param* manifest, int32_t n_params,
             if (opts && opts->grid_blocks > 0)
                 P->grid_blocks = P->unpack_grid_blocks = P->verify_grid_blocks = P->reg_pack_grid =
                     P->reg_unpack_grid = P->reg_vunpack_grid = opts->grid_blocks;
-            // Small plans (not an item for every block): smaller items, so that
-            // every block gets a few.  Pack and verifying unpack of 1, 2 and 4 M
-            // elements in turn on GB300: 15.5, 15.9 and 16.9 us with 64 KiB
-            // items, 12.6, 13.8 and 15.5 us with these; of 8 M, where every block
-            // has a 64 KiB item, 20.9 us, and 21.5 with smaller ones.
-            if (!(opts && opts->chunk_bytes) &&
-                stream_bytes(P) < P->chunk_bytes * P->grid_blocks)
-                while (P->chunk_bytes > kMinChunkBytes &&
-                       stream_bytes(P) < kItemsPerBlock * P->chunk_bytes * P->grid_blocks)
-                    P->chunk_bytes /= 2;
+            P->unpack_chunk_bytes = P->chunk_bytes;
+            if (!(opts && opts->chunk_bytes)) {
+                P->chunk_bytes = small_chunk(P, P->grid_blocks);
+                P->unpack_chunk_bytes = small_chunk(P, P->unpack_grid_blocks);
+            }
         }
         if (st == RR_OK) {
             build_tables(P, dst);
