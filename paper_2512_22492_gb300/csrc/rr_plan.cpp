@@ -49,6 +49,15 @@ constexpr int64_t kSmallPlanItems = 2;         // items per block of a small pla
 #ifndef RR_SHORT_ITEM_OVERHEAD
 #define RR_SHORT_ITEM_OVERHEAD 3072
 #endif
+// In a small table an item of any size costs its block about 0.7 us (its part
+// of the producer's path, not hidden behind a full ring), what 32 KiB of
+// traffic do.  Fourteen 22-element items beside one another kept one block for
+// 20 us of a 30 us pack; weighed so, that pack takes 10 us.  The two-layer test
+// model's: 9.3, 9.3, 7.9, 7.4 and 7.6 us with 1, 8, 16, 32 and 64 KiB, its
+// verifying unpack 8.5, 6.5, 6.3 and 6.3 us with 1, 8, 16 and 32 KiB.
+#ifndef RR_FEW_ITEMS_OVERHEAD
+#define RR_FEW_ITEMS_OVERHEAD (32 * 1024)
+#endif
 #ifndef RR_SHORT_ITEM
 #define RR_SHORT_ITEM (16 * 1024)
 #endif
@@ -436,12 +445,13 @@ struct PackWeight {
 
 struct UnpackWeight {
     bool staged;
+    int64_t overhead = kItemOverhead;
     int64_t operator()(const rr_unpack_item& it) const {
         switch (it.kind) {
-            case RR_ITEM_COPY_VEC: return 2 * int64_t(it.nbytes) + kItemOverhead;
+            case RR_ITEM_COPY_VEC: return 2 * int64_t(it.nbytes) + overhead;
             case RR_ITEM_COPY_SCALAR:
-                return 2 * int64_t(it.nbytes) * (staged ? 11 : 20) / 10 + kItemOverhead;
-            default: return int64_t(it.nbytes) + kItemOverhead;
+                return 2 * int64_t(it.nbytes) * (staged ? 11 : 20) / 10 + overhead;
+            default: return int64_t(it.nbytes) + overhead;
         }
     }
 };
@@ -491,10 +501,11 @@ int64_t taper_size(int64_t rem, int64_t unit_weight, int32_t grid) {
 // time let the fast blocks take more of them, and all finish together.  Within
 // a bucket a cut falls after the item that reaches the unit's size, unless
 // less than a quarter unit would be left in the bucket; no unit is empty.
+// `taper` false: every unit of unit_weight.
 template <class Item, class W>
 void bucket_units(const std::vector<Item>& items, const std::vector<uint32_t>& bucket_first,
                   int64_t unit_weight, int32_t grid, std::vector<uint32_t>& first,
-                  std::vector<uint32_t>& bucket_unit, W w) {
+                  std::vector<uint32_t>& bucket_unit, W w, bool taper = true) {
     first.clear();
     bucket_unit.assign(bucket_first.size(), 0);
     int64_t rem = 0;   // weight from the current item to the end of the table
@@ -508,7 +519,7 @@ void bucket_units(const std::vector<Item>& items, const std::vector<uint32_t>& b
         uint32_t i = lo;
         while (i < hi) {
             first.push_back(i);
-            const int64_t size = taper_size(rem, unit_weight, grid);
+            const int64_t size = taper ? taper_size(rem, unit_weight, grid) : unit_weight;
             int64_t cum = 0;
             while (i < hi) {
                 const int64_t wi = w(items[i++]);
@@ -560,18 +571,35 @@ void whole_units(const std::vector<Item>& items, int32_t grid, int64_t unit_weig
     if (first.size() == size_t(grid) + 1) first.push_back(uint32_t(items.size()));
 }
 
-// Claimed-unit weight for a table: one unit per block on a small plan (with
-// some room for the units that a bucket's end cuts short); else about kUnitsPerBlock units per block of the
+// Claimed-unit weight for a table: about kUnitsPerBlock units per block of the
 // grid, none above kUnitWeight (small enough to even out the finish), none
 // below kUnitWeight / 8 (each costs the producer one claim).
 template <class Item, class W>
 int64_t unit_weight_for(const std::vector<Item>& items, int32_t grid, W w) {
     int64_t total = 0;
     for (const Item& it : items) total += w(it);
-    if (small_table(total, grid, kSmallUnitShare))
-        return std::max<int64_t>(8 * 1024, total * 115 / 100 / std::max(1, grid));
     const int64_t per_block = total / (int64_t(kUnitsPerBlock) * std::max(1, grid));
     return std::min(kUnitWeight, std::max(kUnitWeight / 8, per_block));
+}
+
+// The per-bucket units of a table: on a small one no more than the grid has
+// blocks (the smallest size that gives as few, since a bucket's end cuts units
+// short), else claimed ones.
+template <class Item, class W>
+void table_units(const std::vector<Item>& items, const std::vector<uint32_t>& bucket_first,
+                 int32_t grid, bool small, std::vector<uint32_t>& first,
+                 std::vector<uint32_t>& bucket_unit, W w) {
+    if (small) {
+        int64_t total = 0;
+        for (const Item& it : items) total += w(it);
+        for (int64_t pct = 100; pct <= 200; pct += 5) {
+            bucket_units(items, bucket_first,
+                         std::max<int64_t>(1, total * pct / 100 / std::max(1, grid)), grid, first,
+                         bucket_unit, w, false);
+            if (int64_t(first.size()) - 1 <= grid) return;
+        }
+    }
+    bucket_units(items, bucket_first, unit_weight_for(items, grid, w), grid, first, bucket_unit, w);
 }
 
 rr_status validate_and_describe(rr_plan* P, const rr_param* manifest, int32_t n_params,
@@ -829,7 +857,7 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
     Builder b(P);
     const bool staged = P->engine == RR_ENGINE_AUTO;
     PackWeight pack_weight{staged};
-    const UnpackWeight unpack_weight{staged};
+    UnpackWeight unpack_weight{staged};
     std::vector<std::vector<int32_t>> member;
     const std::vector<FanGroup> groups = find_fan_groups(P, dst, member);
     std::vector<std::pair<size_t, size_t>> fanned;   // regular items of grouped blocks
@@ -894,6 +922,16 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
     const bool short_items =
         data_bytes < std::min<int64_t>(RR_SHORT_ITEM, P->chunk_bytes / 4) * data_items;
     if (staged && short_items) pack_weight.overhead = RR_SHORT_ITEM_OVERHEAD;
+    auto few_items = [&](const auto& items, int32_t grid, int64_t share, auto w) {
+        int64_t total = 0;
+        for (const auto& it : items) total += w(it);
+        return small_table(total, grid, share) && int64_t(items.size()) < 8 * int64_t(grid);
+    };
+    const bool few_pack = few_items(P->pack_items, P->grid_blocks, kSmallPackShare, pack_weight);
+    const bool few_unpack = few_items(P->unpack_items, P->unpack_grid_blocks, kSmallUnitShare,
+                                      unpack_weight);
+    if (staged && few_pack) pack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
+    if (staged && few_unpack) unpack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
     P->pack_plain = !short_items;
     for (const rr_pack_item& it : P->pack_items)
         if (it.kind == RR_ITEM_F32_SCALAR || it.kind == RR_ITEM_BF16_SCALAR) P->pack_plain = false;
@@ -903,13 +941,10 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
             P->unpack_plain = false;
     partition(P->pack_items, P->grid_blocks, P->pack_block_first, pack_weight);
     partition(P->unpack_items, P->unpack_grid_blocks, P->unpack_block_first, unpack_weight);
-    bucket_units(P->unpack_items, P->unpack_bucket_first,
-                 unit_weight_for(P->unpack_items, P->unpack_grid_blocks, unpack_weight),
-                 P->unpack_grid_blocks, P->unpack_unit_first, P->unpack_bucket_unit,
-                 unpack_weight);
-    bucket_units(P->pack_items, P->pack_bucket_first,
-                 unit_weight_for(P->pack_items, P->grid_blocks, pack_weight), P->grid_blocks,
-                 P->pack_unit_first, P->pack_bucket_unit, pack_weight);
+    table_units(P->unpack_items, P->unpack_bucket_first, P->unpack_grid_blocks, few_unpack,
+                P->unpack_unit_first, P->unpack_bucket_unit, unpack_weight);
+    table_units(P->pack_items, P->pack_bucket_first, P->grid_blocks, few_pack, P->pack_unit_first,
+                P->pack_bucket_unit, pack_weight);
     // Summed weights: a register-path call splits its items over the grid by
     // them (and a bulk launch of a bucket range that gets no pooled slot).
     auto prefix = [](const auto& items, std::vector<unsigned long long>& out, auto w) {
