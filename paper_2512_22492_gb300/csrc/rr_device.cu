@@ -1269,24 +1269,25 @@ __device__ __forceinline__ char* bulk_bucket(const BulkArgs<NPTR>& a, uint32_t b
 
 // MODE 0: pack, 1: unpack, 2: unpack with checksum comparison.  CHECK: check
 // every item against the plan's buffers first (the check_items option).  F16
-// (pack only): the rollout's elements are float16, else bfloat16.  FULL: the
-// table may hold elements of any alignment, fan-out heads or runs of short
-// items; the lean kernel (vector items and zero fills alone) has two fifths of
-// the code, and on launches of a few microseconds fetching code counts: a pack
-// and a verifying unpack of 1 K elements in turn take 10.5 us with the full
-// kernels on GB300 and 8.8 us with the lean ones, of 16 M elements 39.4 and
-// 34.2 us.
-template <int NPTR, int MODE, bool CHECK, bool F16, bool FULL>
+// (pack only): the rollout's elements are float16, else bfloat16.  LEVEL: what
+// the table may hold: 0, vector items and zero fills alone; 1 (pack), fan-out
+// heads too; 2, elements of any alignment and runs of short items too.  On
+// launches of a few microseconds fetching code counts, and the lean kernel has
+// two fifths of the full one's: a pack and a verifying unpack of 1 K elements in
+// turn take 10.5 us with the full kernels on GB300 and 8.8 us with the lean
+// ones, of 16 M elements 39.4 and 34.2 us.
+template <int NPTR, int MODE, bool CHECK, bool F16, int LEVEL>
 __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(const __grid_constant__ BulkArgs<NPTR> a) {
     static_assert(MODE == 0 || !F16, "the destination type matters to the pack only");
     using D = DstCast<F16>;
+    constexpr bool FAN = MODE == 0 && LEVEL >= 1, FULL = LEVEL == 2;
     constexpr int kConsumerWarps = BulkShape<MODE>::kWarps;
     constexpr int kStageBytes = BulkShape<MODE>::kStageBytes;
     constexpr int kStages = BulkShape<MODE>::kStages;
     extern __shared__ __align__(128) char stage_mem[];
     __shared__ __align__(8) uint64_t full[kStages], empty[kStages];
     __shared__ Piece meta[kStages];
-    __shared__ rr_pack_item fan_dst[MODE == 0 && FULL ? kStages : 1][kMaxFanDst];   // PC_FAN slices
+    __shared__ rr_pack_item fan_dst[FAN ? kStages : 1][kMaxFanDst];   // PC_FAN slices
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr bool kSum = MODE != 1;
 
@@ -1342,7 +1343,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
             if constexpr (MODE == 0) {
                 // A fan-out piece carries its destination items in shared memory
                 // (each lane's from registers: loaded once per head, not per piece).
-                if (FULL && p.kind == PC_FAN && lane < p.n) fan_dst[s][lane] = fan_mine;
+                if (FAN && p.kind == PC_FAN && lane < p.n) fan_dst[s][lane] = fan_mine;
             }
             const uint32_t stage = smem_u32(stage_mem + s * kStageBytes);
             const uint32_t row_bytes = p.row_len * p.es;
@@ -1541,7 +1542,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                 off = d.dst_off;
                 p.es = (uint16_t)es;
                 p.sum_bucket = d.bucket;
-                if (FULL && (d.kind == RR_ITEM_FAN_F32 || d.kind == RR_ITEM_FAN_BF16)) {
+                if (FAN && (d.kind == RR_ITEM_FAN_F32 || d.kind == RR_ITEM_FAN_BF16)) {
                     // Whole rows of the slices' span, staged once; the destination
                     // items that follow the head are read by the consumers.
                     const uint32_t rb = L * es, nd = d.dst_off;
@@ -1663,7 +1664,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
                 p.src = src + r * sstride + (uint64_t)c * p.es;
                 p.dst = dst ? dst + 2ull * ((uint64_t)r * L + c) : nullptr;
                 p.sum_off = off + 2u * (r * L + c);
-                if (MODE == 0 && FULL && fan) {
+                if (FAN && fan) {
                     p.n = fan;
                     p.sum_off = r;   // first row of this piece within the item
                 }
@@ -1771,7 +1772,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
             }
                 break;
             case PC_FAN:   // pack only
-                if constexpr (MODE == 0 && FULL) {
+                if constexpr (FAN) {
                     // Units of work: each slice's 16-byte output vectors in q parts
                     // (q spreads the slices over all consumer warps, whatever the
                     // number of rows staged); one warp per unit.  nd <= kMaxFanDst
@@ -1840,7 +1841,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
         if (lane == 0) mbar_arrive(smem_u32(&empty[s]));
     }
     if (kSum && cur != 0xFFFFFFFFu) flush(a.sums + (cur - sum_base), acc);
-    if constexpr (MODE == 0 && FULL) {
+    if constexpr (FAN) {
 #pragma unroll
         for (uint32_t j = 0; j < kFanSlots; ++j)
             if (fan_bucket[j] != 0xFFFFFFFFu) flush(a.sums + fan_bucket[j], fan_acc[j]);
@@ -1891,9 +1892,9 @@ __global__ void rr_wait_selftest_kernel(unsigned int* err) {
     if (threadIdx.x == 0) mbar_wait(smem_u32(&bar), 0, err);
 }
 
-template <int NPTR, int MODE, bool CHECK = false, bool F16 = false, bool FULL = true>
+template <int NPTR, int MODE, bool CHECK = false, bool F16 = false, int LEVEL = 2>
 cudaError_t bulk_prepare() {
-    return cudaFuncSetAttribute(rr_bulk_kernel<NPTR, MODE, CHECK, F16, FULL>,
+    return cudaFuncSetAttribute(rr_bulk_kernel<NPTR, MODE, CHECK, F16, LEVEL>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 BulkShape<MODE>::kSmem);
 }
@@ -2291,12 +2292,12 @@ struct BulkOpts {
     bool result_err = false;              //   and the plan's error word after them
 };
 
-template <int NPTR, int MODE, bool CHECK, bool F16, bool FULL>
+template <int NPTR, int MODE, bool CHECK, bool F16, int LEVEL>
 cudaError_t launch_bulk_kernel(rr_plan* P, int32_t grid, cudaStream_t s, const BulkArgs<NPTR>& a) {
     // Once per plan and kernel (its device's context keeps the attribute).
-    constexpr uint64_t bit = 1ull << (16 * MODE + 8 * FULL + 4 * CHECK + 2 * F16 + (NPTR == kLargePtrs));
+    constexpr uint64_t bit = 1ull << (16 * MODE + 4 * (CHECK ? 3 : LEVEL) + 2 * F16 + (NPTR == kLargePtrs));
     if (!(P->prepared.load(std::memory_order_relaxed) & bit)) {
-        const cudaError_t e = bulk_prepare<NPTR, MODE, CHECK, F16, FULL>();
+        const cudaError_t e = bulk_prepare<NPTR, MODE, CHECK, F16, LEVEL>();
         if (e != cudaSuccess) return e;
         P->prepared.fetch_or(bit, std::memory_order_relaxed);
     }
@@ -2313,18 +2314,20 @@ cudaError_t launch_bulk_kernel(rr_plan* P, int32_t grid, cudaStream_t s, const B
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, rr_bulk_kernel<NPTR, MODE, CHECK, F16, FULL>, a);
+    return cudaLaunchKernelEx(&cfg, rr_bulk_kernel<NPTR, MODE, CHECK, F16, LEVEL>, a);
 }
 
 // The instantiation for a launch.  The checked kernels (a debugging aid) exist
 // with the large pointer table and the full code only.
 template <int NPTR, int MODE, bool F16>
-cudaError_t launch_bulk_kernel(rr_plan* P, bool full, int32_t grid, cudaStream_t s,
+cudaError_t launch_bulk_kernel(rr_plan* P, int level, int32_t grid, cudaStream_t s,
                                const BulkArgs<NPTR>& a) {
     if constexpr (NPTR == kLargePtrs)
-        if (P->check_items) return launch_bulk_kernel<NPTR, MODE, true, F16, true>(P, grid, s, a);
-    return full ? launch_bulk_kernel<NPTR, MODE, false, F16, true>(P, grid, s, a)
-                : launch_bulk_kernel<NPTR, MODE, false, F16, false>(P, grid, s, a);
+        if (P->check_items) return launch_bulk_kernel<NPTR, MODE, true, F16, 2>(P, grid, s, a);
+    if constexpr (MODE == 0)
+        if (level == 1) return launch_bulk_kernel<NPTR, MODE, false, F16, 1>(P, grid, s, a);
+    return level == 0 ? launch_bulk_kernel<NPTR, MODE, false, F16, 0>(P, grid, s, a)
+                      : launch_bulk_kernel<NPTR, MODE, false, F16, 2>(P, grid, s, a);
 }
 
 template <int NPTR, int MODE>
@@ -2420,11 +2423,12 @@ rr_status launch_bulk(const rr_plan* P, Range R, const void* const* src_shards,
     }
     // The float16 instantiations exist for the pack only (F16 = MODE == 0 there).
     constexpr bool kF16 = MODE == 0;
-    const bool full = MODE == 0 ? (a.items == P->d_full_items || !P->pack_plain)
-                                : !P->unpack_plain;
+    const int level = !(MODE == 0 ? P->pack_plain : P->unpack_plain) ? 2
+                      : MODE == 0 && a.items == P->d_full_items     ? 1
+                                                                    : 0;
     const cudaError_t e = MODE == 0 && P->dst_f16
-                              ? launch_bulk_kernel<NPTR, MODE, kF16>(M, full, grid, s, a)
-                              : launch_bulk_kernel<NPTR, MODE, false>(M, full, grid, s, a);
+                              ? launch_bulk_kernel<NPTR, MODE, kF16>(M, level, grid, s, a)
+                              : launch_bulk_kernel<NPTR, MODE, false>(M, level, grid, s, a);
     if (e != cudaSuccess) return cuda_fail(e, "bulk kernel launch");
     if (slot >= 0) M->slot_seq[slot] = a.end.seq;
     return RR_OK;
@@ -2795,10 +2799,10 @@ rr_status rr_device_default_grid(rr_grids* g) {
     int bp = 0;
     RR_CUDA((bulk_prepare<kLargePtrs, 0>()));
     RR_CUDA((bulk_prepare<kLargePtrs, 2>()));
-    RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bp, rr_bulk_kernel<kLargePtrs, 0, false, false, true>,
+    RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bp, rr_bulk_kernel<kLargePtrs, 0, false, false, 2>,
                                                           BulkShape<0>::kThreads,
                                                           BulkShape<0>::kSmem));
-    RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, rr_bulk_kernel<kLargePtrs, 2, false, false, true>,
+    RR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, rr_bulk_kernel<kLargePtrs, 2, false, false, 2>,
                                                           BulkShape<2>::kThreads,
                                                           BulkShape<2>::kSmem));
     g->reg_pack = sms * (p > 0 ? p : 1);

@@ -933,8 +933,6 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
     if (staged && few_pack) pack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
     if (staged && few_unpack) unpack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
     P->pack_plain = !short_items;
-    for (const rr_pack_item& it : P->pack_items)
-        if (it.kind == RR_ITEM_F32_SCALAR || it.kind == RR_ITEM_BF16_SCALAR) P->pack_plain = false;
     P->unpack_plain = true;
     for (const rr_unpack_item& it : P->unpack_items)
         if (it.kind == RR_ITEM_COPY_SCALAR || it.kind == RR_ITEM_READ_SCALAR)
@@ -1003,6 +1001,11 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
             while (f[g] < P->full_items.size() && P->full_items[f[g]].kind == RR_ITEM_FAN_DST) ++f[g];
         }
     }
+
+    for (const std::vector<rr_pack_item>* items : {&P->pack_items, &P->full_items})
+        for (const rr_pack_item& it : *items)
+            if (it.kind == RR_ITEM_F32_SCALAR || it.kind == RR_ITEM_BF16_SCALAR)
+                P->pack_plain = false;
 
     // Units of a pack over every bucket.
     const std::vector<rr_pack_item>& whole = P->full_items.empty() ? P->pack_items : P->full_items;
