@@ -2633,10 +2633,13 @@ rr_status unpack_impl(const rr_plan* P, Range R, const void* const* buckets, voi
 rr_status read_error(const rr_plan* P, cudaStream_t stream);
 
 // The answer of a blocking verify: its last launch's last block writes it to
-// the plan's pinned words, with the plan's error word as it then is.
+// the plan's pinned words, with the plan's error word (32 bits) as it then is.
+constexpr unsigned long long kNoAnswer = ~0ull;   // in the error word's place before that
 rr_status read_result(const rr_plan* P, int64_t* n_bad, int64_t* first_bad, cudaStream_t stream) {
     RR_CUDA(cudaStreamSynchronize(stream));
-    const long long* h = (const long long*)P->h_verify_result;
+    const volatile long long* h = (const volatile long long*)P->h_verify_result;
+    if ((unsigned long long)h[2] == kNoAnswer)
+        return rr_fail(RR_ECUDA, "the verify's launch ended without an answer");
     if (h[2]) {
         rr_status st = read_error(P, stream);
         if (st) return st;
@@ -2715,6 +2718,7 @@ rr_status unpack_verify_impl(const rr_plan* P, Range R, const void* const* bucke
     if (R.b1 == R.b0) return RR_OK;
     rr_plan* M = const_cast<rr_plan*>(P);   // the scratch area is the only mutable state
     std::lock_guard<std::mutex> lock(M->verify_mutex);
+    P->h_verify_result[2] = kNoAnswer;
     if ((st = enqueue_unpack_verify(P, R, buckets, checksums, dst, bad, on_device, stream,
                                     (long long*)P->h_verify_result)))
         return st;
@@ -2757,6 +2761,7 @@ rr_status verify_impl(const rr_plan* P, Range R, const void* const* buckets,
 
     rr_plan* M = const_cast<rr_plan*>(P);   // the scratch area is the only mutable state
     std::lock_guard<std::mutex> lock(M->verify_mutex);
+    P->h_verify_result[2] = kNoAnswer;
     const int32_t n = R.b1 - R.b0;
     // Separately allocated buckets: one launch per run of buckets that fits the
     // pointer table, sharing the call's counters (ticket reset in between).
