@@ -2150,11 +2150,14 @@ rr_status launch_unpack(const rr_plan* P, Range R, const void* const* buckets, v
 }
 
 // Bytes per chunk of a verify: kVerifyChunk, less where that would leave blocks
-// without one.
+// without one, but at least what a block has in flight (a 4 MiB verify's kernel
+// takes 7.9 us with 16 KiB chunks on GB300, 9.0 with 64 KiB, 9.2 with 8 KiB).
 uint64_t verify_chunk(uint64_t bucket_bytes, uint64_t n, int32_t grid) {
-    const uint64_t share = (bucket_bytes * n / (uint64_t)std::max(1, grid) + 4095) / 4096 * 4096;
+    constexpr uint64_t kLeast = 16ull * kThreads * kUnroll;
+    const uint64_t share =
+        (bucket_bytes * n / (uint64_t)std::max(1, grid) + kLeast - 1) / kLeast * kLeast;
     return std::min(bucket_bytes,
-                    std::min<uint64_t>(kVerifyChunk, std::max<uint64_t>(4096, share)));
+                    std::min<uint64_t>(kVerifyChunk, std::max<uint64_t>(kLeast, share)));
 }
 
 template <int NPTR>
