@@ -58,6 +58,9 @@ constexpr int64_t kSmallPlanItems = 2;         // items per block of a small pla
 #ifndef RR_FEW_ITEMS_OVERHEAD
 #define RR_FEW_ITEMS_OVERHEAD (32 * 1024)
 #endif
+#ifndef RR_FEW_ITEMS_PER_BLOCK
+#define RR_FEW_ITEMS_PER_BLOCK 8
+#endif
 #ifndef RR_SHORT_ITEM
 #define RR_SHORT_ITEM (16 * 1024)
 #endif
@@ -475,11 +478,21 @@ void partition(const std::vector<Item>& items, int32_t grid, std::vector<uint32_
 // microseconds, which every claim (a round trip to L2) would only lengthen: its
 // blocks get all of their work up front.  Measured on GB300: the pack of 8 M
 // elements (330 KiB a block) 14.8 us with claims, 11.7 without, of 16 M 20.6 and
-// 20.1; the verifying unpack (two blocks per SM) of 8 M (110 KiB a block) the
-// same, of 64 M (880 KiB) 45.0 and 45.8.
+// 20.1, of 20 M 27.3 and 25.9, of 23 M (920 KiB) 29.2 and 27.2, of 25 M (1000
+// KiB) 32.4 and 32.5; the verifying unpack (two blocks per SM) of 8 M (110 KiB a
+// block) the same, of 64 M (880 KiB) 45.0 and 45.8.  With half of these limits
+// twelve packs and unpacks of 11 to 32 M elements took 2 to 14% more (19 M bf16,
+// 510 KiB a block: 13.4 us for 11.6), three 2 to 5% less (17 M fp32: 24.1, 25.3).
 constexpr int64_t kSmallPackShare = 1024 * 1024, kSmallUnitShare = 256 * 1024;
 bool small_table(int64_t total, int32_t grid, int64_t share) {
     return total < share * std::max(1, grid);
+}
+
+template <class Item, class W>
+int64_t total_weight(const std::vector<Item>& items, W w) {
+    int64_t total = 0;
+    for (const Item& it : items) total += w(it);
+    return total;
 }
 
 // Claimed units get smaller toward the end of the table (guided
@@ -535,17 +548,17 @@ void bucket_units(const std::vector<Item>& items, const std::vector<uint32_t>& b
 }
 
 // Units for a launch over every bucket (the table it runs is fixed): blocks
-// first drain kOwnShare of the table's weight in equal contiguous shares (unit
-// g < grid is block g's own: no claims, long runs), then claim units of
-// taper_size over the rest.  Own units may be empty.  A cut never falls before
-// a fan-out destination item (a head and its destinations stay in one unit).
+// first drain kOwnShare of the table's weight (a small table's: all of it) in
+// equal contiguous shares (unit g < grid is block g's own: no claims, long
+// runs), then claim units of taper_size over the rest.  Own units may be empty.
+// A cut never falls before a fan-out destination item (a head and its
+// destinations stay in one unit).
 constexpr int64_t kOwnShareNum = RR_OWN_SHARE_PCT, kOwnShareDen = 100;
 template <class Item, class W>
-void whole_units(const std::vector<Item>& items, int32_t grid, int64_t unit_weight,
+void whole_units(const std::vector<Item>& items, int32_t grid, int64_t unit_weight, bool small,
                  std::vector<uint32_t>& first, W w) {
-    int64_t total = 0;
-    for (const Item& it : items) total += w(it);
-    const int64_t own = small_table(total, grid, kSmallPackShare) ? total : total * kOwnShareNum / kOwnShareDen;
+    const int64_t total = total_weight(items, w);
+    const int64_t own = small ? total : total * kOwnShareNum / kOwnShareDen;
     first.assign(size_t(grid) + 1, uint32_t(items.size()));
     first[0] = 0;
     int64_t cum = 0;
@@ -576,8 +589,7 @@ void whole_units(const std::vector<Item>& items, int32_t grid, int64_t unit_weig
 // below kUnitWeight / 8 (each costs the producer one claim).
 template <class Item, class W>
 int64_t unit_weight_for(const std::vector<Item>& items, int32_t grid, W w) {
-    int64_t total = 0;
-    for (const Item& it : items) total += w(it);
+    const int64_t total = total_weight(items, w);
     const int64_t per_block = total / (int64_t(kUnitsPerBlock) * std::max(1, grid));
     return std::min(kUnitWeight, std::max(kUnitWeight / 8, per_block));
 }
@@ -590,8 +602,7 @@ void table_units(const std::vector<Item>& items, const std::vector<uint32_t>& bu
                  int32_t grid, bool small, std::vector<uint32_t>& first,
                  std::vector<uint32_t>& bucket_unit, W w) {
     if (small) {
-        int64_t total = 0;
-        for (const Item& it : items) total += w(it);
+        const int64_t total = total_weight(items, w);
         for (int64_t pct = 100; pct <= 200; pct += 5) {
             bucket_units(items, bucket_first,
                          std::max<int64_t>(1, total * pct / 100 / std::max(1, grid)), grid, first,
@@ -922,14 +933,18 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
     const bool short_items =
         data_bytes < std::min<int64_t>(RR_SHORT_ITEM, P->chunk_bytes / 4) * data_items;
     if (staged && short_items) pack_weight.overhead = RR_SHORT_ITEM_OVERHEAD;
-    auto few_items = [&](const auto& items, int32_t grid, int64_t share, auto w) {
-        int64_t total = 0;
-        for (const auto& it : items) total += w(it);
-        return small_table(total, grid, share) && int64_t(items.size()) < 8 * int64_t(grid);
+    // Whether a table is small is decided once, on the weights from before the
+    // raise below.
+    auto few = [](const auto& items, int32_t grid) {
+        return int64_t(items.size()) < RR_FEW_ITEMS_PER_BLOCK * int64_t(grid);
     };
-    const bool few_pack = few_items(P->pack_items, P->grid_blocks, kSmallPackShare, pack_weight);
-    const bool few_unpack = few_items(P->unpack_items, P->unpack_grid_blocks, kSmallUnitShare,
-                                      unpack_weight);
+    const PackWeight traffic = pack_weight;
+    const bool few_pack = small_table(total_weight(P->pack_items, traffic), P->grid_blocks,
+                                      kSmallPackShare) &&
+                          few(P->pack_items, P->grid_blocks);
+    const bool few_unpack = small_table(total_weight(P->unpack_items, unpack_weight),
+                                        P->unpack_grid_blocks, kSmallUnitShare) &&
+                            few(P->unpack_items, P->unpack_grid_blocks);
     if (staged && few_pack) pack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
     if (staged && few_unpack) unpack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
     P->pack_plain = !short_items;
@@ -1010,6 +1025,7 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
     // Units of a pack over every bucket.
     const std::vector<rr_pack_item>& whole = P->full_items.empty() ? P->pack_items : P->full_items;
     whole_units(whole, P->grid_blocks, unit_weight_for(whole, P->grid_blocks, pack_weight),
+                small_table(total_weight(whole, traffic), P->grid_blocks, kSmallPackShare),
                 P->pack_whole_unit_first, pack_weight);
 
     rr_plan_stats& s = P->stats;

@@ -42,3 +42,21 @@ def test_small_plan_tables(name, grid):
         got = U.check_and_run_pack(table, shards, plan.n_buckets, plan.bucket_bytes,
                                    plan.shard_bytes)
         np.testing.assert_array_equal(got, want)
+
+
+@pytest.mark.parametrize("mi", [8, 20, 22, 24, 25, 26, 28, 40])
+def test_small_tables_are_told_by_their_traffic(mi):
+    """Under 1 MiB of traffic a block every unit of the whole-sync pack is a
+    block's own; from there on 15% of the table's weight is left to claim.  An
+    item weighs 1 KiB beyond its bytes where this is decided, whatever it weighs
+    in the split that follows."""
+    n, grid = mi << 20, 152
+    plan = rr.rr_plan_create([rr.Param("a", (n,), "f32")], rr.SrcLayout(1),
+                             rr.DstLayout(1, [rr.DstTensor("t", 0, [rr.Block(0, 0, n, 0, 1)])]),
+                             1 << 20, rr.PlanOptions(host_only=True, grid_blocks=grid))
+    full, _ = plan.export_pack_full()
+    whole, _ = U.check_units(plan, len(full), "pack_full")
+    small = 6 * n + 1024 * len(full) < (grid << 20)
+    assert small == (mi < 26)
+    own = whole[grid] / len(full)
+    assert own == 1 if small else 0.8 < own < 0.9
