@@ -141,10 +141,11 @@ struct UnpackArgs {
     uint64_t bucket_stride;
     int32_t dst_base;         // index in ptr[] of destination tensor 0
     int32_t bucket_lo;        // table mode: the first bucket the table holds
-    // Claimed work units (claim NULL: none, the split above).  unit_first holds
-    // the first item of each of n_units units and one past the last; block g
-    // walks unit g, then claims the next unclaimed unit (atomicAdd on *claim,
-    // zero at launch) until none are left.  claim is end.counters + 3.
+    // Work units (n_units 0: none, the split above).  unit_first holds the first
+    // item of each of n_units units and one past the last; block g walks unit g,
+    // then claims the next unclaimed unit (atomicAdd on *claim, zero at launch)
+    // until none are left.  claim is end.counters + 3, or NULL: every block
+    // walks an equal run of the units.
     const uint32_t* unit_first;
     unsigned long long* claim;
     uint32_t n_units;
@@ -360,8 +361,6 @@ __device__ __forceinline__ bool unpack_item_ok(const ItemBounds& b, const rr_unp
     return ok;
 }
 
-// This block's item range: the plan's balanced split for a full call, an even
-// split of [begin, end) for a bucket-range call.
 // First item i in [lo, hi] with prefix[i] >= w (prefix is non-decreasing).
 __device__ __forceinline__ uint32_t lower_item(const unsigned long long* prefix, uint32_t lo,
                                                uint32_t hi, unsigned long long w) {
@@ -375,6 +374,8 @@ __device__ __forceinline__ uint32_t lower_item(const unsigned long long* prefix,
     return lo;
 }
 
+// This block's item range: the plan's balanced split for a full call, an even
+// split of [begin, end) for a bucket-range call.
 __device__ __forceinline__ void block_items(const uint32_t* block_first,
                                             const unsigned long long* prefix, uint32_t begin,
                                             uint32_t end, uint32_t* i0, uint32_t* i1) {
@@ -395,6 +396,14 @@ __device__ __forceinline__ void block_items(const uint32_t* block_first,
         *i0 = begin + (uint32_t)(n * blockIdx.x / gridDim.x);
         *i1 = begin + (uint32_t)(n * (blockIdx.x + 1) / gridDim.x);
     }
+}
+
+// This block's equal run of n unclaimed units (the first blocks take one more).
+__device__ __forceinline__ void block_units(const uint32_t* first, uint32_t n, uint32_t* i0,
+                                            uint32_t* i1) {
+    const uint32_t q = n / gridDim.x, more = n - q * gridDim.x, g = blockIdx.x;
+    *i0 = first[q * g + min(g, more)];
+    *i1 = first[q * (g + 1) + min(g + 1, more)];
 }
 
 template <int NPTR>
@@ -687,7 +696,10 @@ __global__ void __launch_bounds__(RegUnpackShape<VERIFY>::kBlock, 4) rr_unpack_k
     uint32_t walked = 0;              // units this block has walked
     unsigned long long pending = 0;   // thread 0: the claim in flight
     if (!a.claim) {
-        block_items(a.block_first, a.weight_prefix, a.item_begin, a.item_end, &i0, &i1);
+        if (a.n_units)
+            block_units(a.unit_first, a.n_units, &i0, &i1);
+        else
+            block_items(a.block_first, a.weight_prefix, a.item_begin, a.item_end, &i0, &i1);
     } else {
         if (blockIdx.x < a.n_units) {
             i0 = a.unit_first[blockIdx.x];
@@ -916,10 +928,11 @@ struct BulkArgs {
     int32_t first_bucket;        // the call's range [first_bucket, first_bucket + n_buckets)
     int32_t n_buckets;
     unsigned int* err;
-    // Claimed work units (NULL: none).  block_first then holds the first item
-    // of each of n_units units (and one past the last): unit g < gridDim.x is
-    // block g's own, the rest go to whichever block asks next (atomicAdd on
-    // *claim = end.counters[3], zero at launch).
+    // Work units (n_units 0: none).  block_first then holds the first item of
+    // each of n_units units (and one past the last): unit g < gridDim.x is block
+    // g's own, the rest go to whichever block asks next (atomicAdd on *claim =
+    // end.counters[3], zero at launch).  claim NULL: every block takes an equal
+    // run of the units.
     unsigned long long* claim;
     uint32_t n_units;
     uint32_t pad2_;
@@ -1308,9 +1321,12 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1) rr_bulk_kernel(c
 
     // The plan's tables are immutable: read them before the wait.
     uint32_t i0 = 0, i1 = 0;
-    if (!a.claim)
-        block_items(a.block_first, a.weight_prefix, a.item_begin, a.item_end, &i0, &i1);
-    else if (blockIdx.x < a.n_units) {
+    if (!a.claim) {
+        if (a.n_units)
+            block_units(a.block_first, a.n_units, &i0, &i1);
+        else
+            block_items(a.block_first, a.weight_prefix, a.item_begin, a.item_end, &i0, &i1);
+    } else if (blockIdx.x < a.n_units) {
         i0 = a.block_first[blockIdx.x];
         i1 = a.block_first[blockIdx.x + 1];
     }
@@ -2037,8 +2053,8 @@ ItemBounds bounds_of(const rr_plan* P) {
 }
 
 int32_t take_slot(rr_plan* M, cudaStream_t s, LaunchEnd* end);
-template <int MODE>
-void work_units(const rr_plan* P, const Range& R, const uint32_t** first, uint32_t* n);
+template <int MODE, class Args>
+void set_units(const rr_plan* P, const Range& R, Args& a, const uint32_t** first);
 
 // The register-path pack instantiation for a launch: item checks, a source in
 // host memory, and the destination type.
@@ -2126,14 +2142,10 @@ rr_status launch_unpack(const rr_plan* P, Range R, const void* const* buckets, v
     std::unique_lock<std::mutex> lock(M->claim_mutex, std::defer_lock);
     int32_t slot = -1;
     if (checksums) {
-        a.claim = a.end.counters + 3;
-        work_units<1>(P, R, &a.unit_first, &a.n_units);
+        set_units<1>(P, R, a, &a.unit_first);
     } else {
         lock.lock();
-        if ((slot = take_slot(M, s, &a.end)) >= 0) {
-            a.claim = a.end.counters + 3;
-            work_units<1>(P, R, &a.unit_first, &a.n_units);
-        }
+        if ((slot = take_slot(M, s, &a.end)) >= 0) set_units<1>(P, R, a, &a.unit_first);
     }
     constexpr int VT = RegUnpackShape<true>::kBlock;
     if (checksums && P->check_items)
@@ -2266,24 +2278,42 @@ int32_t take_slot(rr_plan* M, cudaStream_t s, LaunchEnd* end) {
     return slot;
 }
 
-// The work units of a bulk launch over range R: for a pack over every bucket
-// the whole table's (own shares, then claimed), else the per-bucket units of
-// R's buckets (all claimed).  Measured on GB300: the fp32 pack (2 bytes read
-// per byte written) runs best with long own runs; the 1:1 unpack passes best
-// with every unit claimed.
+// The work units of a launch over range R, and whether they are claimed: for a
+// pack over every bucket the whole table's (own shares, then claimed), else the
+// per-bucket units of R's buckets (all claimed).  Measured on GB300: the fp32
+// pack (2 bytes read per byte written) runs best with long own runs; the 1:1
+// unpack passes best with every unit claimed.  A small table's are not claimed:
+// every block takes an equal run of them.
+struct Units {
+    const uint32_t* first;
+    uint32_t n;
+    bool claimed;
+};
 template <int MODE>
-void work_units(const rr_plan* P, const Range& R, const uint32_t** first, uint32_t* n) {
+Units work_units(const rr_plan* P, const Range& R) {
     if (MODE == 0 && R.full) {
-        *first = P->d_pack_whole_unit_first;
-        *n = uint32_t(P->pack_whole_unit_first.size() - 1);
-        if (*n == uint32_t(P->grid_blocks) + 1 &&   // no claimed unit that holds an item
-            P->pack_whole_unit_first[*n - 1] == P->pack_whole_unit_first[*n])
-            --*n;
-    } else {
-        const std::vector<uint32_t>& bu = MODE == 0 ? P->pack_bucket_unit : P->unpack_bucket_unit;
-        *first = (MODE == 0 ? P->d_pack_unit_first : P->d_unpack_unit_first) + bu[R.b0];
-        *n = bu[R.b1] - bu[R.b0];
+        uint32_t n = uint32_t(P->pack_whole_unit_first.size() - 1);
+        if (n == uint32_t(P->grid_blocks) + 1 &&   // no claimed unit that holds an item
+            P->pack_whole_unit_first[n - 1] == P->pack_whole_unit_first[n])
+            --n;
+        return {P->d_pack_whole_unit_first, n, n > uint32_t(P->grid_blocks)};
     }
+    if (MODE != 0 && P->unpack_small && R.b0 == 0 && R.b1 == P->n_buckets)
+        return {P->d_unpack_whole_unit_first, uint32_t(P->unpack_whole_unit_first.size() - 1), false};
+    const std::vector<uint32_t>& bu = MODE == 0 ? P->pack_bucket_unit : P->unpack_bucket_unit;
+    return {(MODE == 0 ? P->d_pack_unit_first : P->d_unpack_unit_first) + bu[R.b0],
+            bu[R.b1] - bu[R.b0], !(MODE == 0 ? P->pack_small : P->unpack_small)};
+}
+
+// Gives a launch its units; claimed ones through the counter among the call's or
+// the slot's (a.end).
+template <int MODE, class Args>
+void set_units(const rr_plan* P, const Range& R, Args& a, const uint32_t** first) {
+    const Units u = work_units<MODE>(P, R);
+    if (!u.n) return;
+    *first = u.first;
+    a.n_units = u.n;
+    a.claim = u.claimed ? a.end.counters + 3 : nullptr;
 }
 
 // How a bulk launch may use the plan's pooled slots, and what it zeroes itself.
@@ -2397,8 +2427,7 @@ rr_status launch_bulk(const rr_plan* P, Range R, const void* const* src_shards,
     }
     if (slot >= 0) {
         unsigned long long* area = a.end.counters - P->n_buckets;
-        a.claim = a.end.counters + 3;
-        work_units<MODE>(P, R, &a.block_first, &a.n_units);
+        set_units<MODE>(P, R, a, &a.block_first);
         if (MODE == 0 && o.zero) {          // the checksums come out of the slot's sums
             a.sums = area;
             a.sums_out = (unsigned long long*)checksums;
@@ -2413,9 +2442,8 @@ rr_status launch_bulk(const rr_plan* P, Range R, const void* const* src_shards,
             const SumSlot q = sum_slot(P, R, bad);
             a.sums = q.sums;
             a.end.counters = q.counters;
-            a.claim = q.counters + 3;       // the call's work units, claimed through counters[3]
             a.bad = q.bad;
-            work_units<MODE>(P, R, &a.block_first, &a.n_units);
+            set_units<MODE>(P, R, a, &a.block_first);
         }
     }
     if (MODE == 2) {
@@ -2848,6 +2876,8 @@ rr_status rr_device_upload(rr_plan* P) {
                 P->unpack_block_first.size() * sizeof(uint32_t))) != cudaSuccess ||
         (e = up((void**)&P->d_unpack_unit_first, P->unpack_unit_first.data(),
                 P->unpack_unit_first.size() * sizeof(uint32_t))) != cudaSuccess ||
+        (e = up((void**)&P->d_unpack_whole_unit_first, P->unpack_whole_unit_first.data(),
+                P->unpack_whole_unit_first.size() * sizeof(uint32_t))) != cudaSuccess ||
         (e = up((void**)&P->d_pack_unit_first, P->pack_unit_first.data(),
                 P->pack_unit_first.size() * sizeof(uint32_t))) != cudaSuccess ||
         (e = up((void**)&P->d_pack_whole_unit_first, P->pack_whole_unit_first.data(),
@@ -2903,6 +2933,7 @@ void rr_device_release(rr_plan* P) {
     cudaFree(P->d_unpack_items);
     cudaFree(P->d_unpack_block_first);
     cudaFree(P->d_unpack_unit_first);
+    cudaFree(P->d_unpack_whole_unit_first);
     cudaFree(P->d_pack_unit_first);
     cudaFree(P->d_pack_whole_unit_first);
     if (P->slot_copies) {   // a copy of the done words may still be under way
@@ -2926,6 +2957,7 @@ void rr_device_release(rr_plan* P) {
     P->d_unpack_items = nullptr;
     P->d_unpack_block_first = nullptr;
     P->d_unpack_unit_first = nullptr;
+    P->d_unpack_whole_unit_first = nullptr;
     P->d_pack_unit_first = nullptr;
     P->d_pack_whole_unit_first = nullptr;
     P->d_slots = nullptr;

@@ -69,6 +69,7 @@ struct rr_plan {
     // past the last); per bucket, its first unit (n_buckets + 1).
     std::vector<uint32_t> unpack_unit_first;
     std::vector<uint32_t> unpack_bucket_unit;
+    std::vector<uint32_t> unpack_whole_unit_first; // unpack_small: for a call over every bucket
     std::vector<uint32_t> pack_unit_first;
     std::vector<uint32_t> pack_bucket_unit;
     std::vector<uint32_t> pack_whole_unit_first;   // a pack over every bucket: own units
@@ -79,6 +80,8 @@ struct rr_plan {
     std::vector<rr_pack_item> full_items;       // whole-sync table with fan-out groups;
                                                 // empty when it would equal pack_items
     std::vector<uint32_t> full_block_first;     // grid_blocks + 1
+    bool pack_small = false;          // small tables: nothing is claimed, every block takes
+    bool unpack_small = false;        //   an equal run of the launch's units
     bool pack_plain = false;          // pack_items / unpack_items hold vector items and zero
     bool unpack_plain = false;        //   fills alone, no runs of short ones (the lean kernels)
     std::vector<uint32_t> unpack_bucket_first;  // n_buckets + 1: first unpack item of bucket b
@@ -103,6 +106,7 @@ struct rr_plan {
     rr_unpack_item* d_unpack_items = nullptr;
     uint32_t* d_unpack_block_first = nullptr;
     uint32_t* d_unpack_unit_first = nullptr;
+    uint32_t* d_unpack_whole_unit_first = nullptr;
     uint32_t* d_pack_unit_first = nullptr;
     uint32_t* d_pack_whole_unit_first = nullptr;
     // Pooled scratch of launches that need no per-call scratch: a slot is

@@ -61,6 +61,9 @@ constexpr int64_t kSmallPlanItems = 2;         // items per block of a small pla
 #ifndef RR_FEW_ITEMS_PER_BLOCK
 #define RR_FEW_ITEMS_PER_BLOCK 8
 #endif
+#ifndef RR_SMALL_UNITS
+#define RR_SMALL_UNITS 6
+#endif
 #ifndef RR_SHORT_ITEM
 #define RR_SHORT_ITEM (16 * 1024)
 #endif
@@ -594,23 +597,40 @@ int64_t unit_weight_for(const std::vector<Item>& items, int32_t grid, W w) {
     return std::min(kUnitWeight, std::max(kUnitWeight / 8, per_block));
 }
 
-// The per-bucket units of a table: on a small one no more than the grid has
-// blocks (the smallest size that gives as few, since a bucket's end cuts units
-// short), else claimed ones.
+// The per-bucket units of a table: claimed ones, or on a small table (nothing is
+// claimed) RR_SMALL_UNITS for every block of the grid, so that a launch over a
+// range of buckets can give every block an equal run of them.  As few units as
+// blocks, claimed, left most of the grid idle: packing a 16th of the buckets of a
+// 12 M element fp32 plan took 16.4 us on GB300, and half of them 17.9; with these
+// 7.2 and 13.0.  Of 3, 4, 6, 8 and 16 a block 6 had the fewest ranges slower than
+// claimed units of at least 128 KiB (coarse runs leave some blocks one unit more,
+// fine ones cut items of unequal weights).
 template <class Item, class W>
 void table_units(const std::vector<Item>& items, const std::vector<uint32_t>& bucket_first,
                  int32_t grid, bool small, std::vector<uint32_t>& first,
                  std::vector<uint32_t>& bucket_unit, W w) {
-    if (small) {
-        const int64_t total = total_weight(items, w);
-        for (int64_t pct = 100; pct <= 200; pct += 5) {
-            bucket_units(items, bucket_first,
-                         std::max<int64_t>(1, total * pct / 100 / std::max(1, grid)), grid, first,
-                         bucket_unit, w, false);
-            if (int64_t(first.size()) - 1 <= grid) return;
-        }
+    const int64_t unit = small ? std::max<int64_t>(1, total_weight(items, w) /
+                                                          (RR_SMALL_UNITS * int64_t(std::max(1, grid))))
+                               : unit_weight_for(items, grid, w);
+    bucket_units(items, bucket_first, unit, grid, first, bucket_unit, w, !small);
+}
+
+// A small table's units for a launch over every bucket, no more than the grid
+// has blocks: the smallest per-bucket units that give as few (a bucket's end
+// cuts units short), else the balanced ranges `block_first`.
+template <class Item, class W>
+std::vector<uint32_t> small_whole_units(const std::vector<Item>& items,
+                                        const std::vector<uint32_t>& bucket_first, int32_t grid,
+                                        const std::vector<uint32_t>& block_first, W w) {
+    const int64_t total = total_weight(items, w);
+    std::vector<uint32_t> first, bucket_unit;
+    for (int64_t pct = 100; pct <= 200; pct += 5) {
+        bucket_units(items, bucket_first,
+                     std::max<int64_t>(1, total * pct / 100 / std::max(1, grid)), grid, first,
+                     bucket_unit, w, false);
+        if (int64_t(first.size()) - 1 <= grid) return first;
     }
-    bucket_units(items, bucket_first, unit_weight_for(items, grid, w), grid, first, bucket_unit, w);
+    return block_first;
 }
 
 rr_status validate_and_describe(rr_plan* P, const rr_param* manifest, int32_t n_params,
@@ -939,14 +959,13 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
         return int64_t(items.size()) < RR_FEW_ITEMS_PER_BLOCK * int64_t(grid);
     };
     const PackWeight traffic = pack_weight;
-    const bool few_pack = small_table(total_weight(P->pack_items, traffic), P->grid_blocks,
-                                      kSmallPackShare) &&
-                          few(P->pack_items, P->grid_blocks);
-    const bool few_unpack = small_table(total_weight(P->unpack_items, unpack_weight),
-                                        P->unpack_grid_blocks, kSmallUnitShare) &&
-                            few(P->unpack_items, P->unpack_grid_blocks);
-    if (staged && few_pack) pack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
-    if (staged && few_unpack) unpack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
+    P->pack_small = small_table(total_weight(P->pack_items, traffic), P->grid_blocks,
+                                kSmallPackShare) && few(P->pack_items, P->grid_blocks);
+    P->unpack_small = small_table(total_weight(P->unpack_items, unpack_weight),
+                                  P->unpack_grid_blocks, kSmallUnitShare) &&
+                      few(P->unpack_items, P->unpack_grid_blocks);
+    if (staged && P->pack_small) pack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
+    if (staged && P->unpack_small) unpack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
     P->pack_plain = !short_items;
     P->unpack_plain = true;
     for (const rr_unpack_item& it : P->unpack_items)
@@ -954,10 +973,15 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
             P->unpack_plain = false;
     partition(P->pack_items, P->grid_blocks, P->pack_block_first, pack_weight);
     partition(P->unpack_items, P->unpack_grid_blocks, P->unpack_block_first, unpack_weight);
-    table_units(P->unpack_items, P->unpack_bucket_first, P->unpack_grid_blocks, few_unpack,
+    table_units(P->unpack_items, P->unpack_bucket_first, P->unpack_grid_blocks, P->unpack_small,
                 P->unpack_unit_first, P->unpack_bucket_unit, unpack_weight);
-    table_units(P->pack_items, P->pack_bucket_first, P->grid_blocks, few_pack, P->pack_unit_first,
-                P->pack_bucket_unit, pack_weight);
+    P->unpack_whole_unit_first.clear();
+    if (P->unpack_small)
+        P->unpack_whole_unit_first =
+            small_whole_units(P->unpack_items, P->unpack_bucket_first, P->unpack_grid_blocks,
+                              P->unpack_block_first, unpack_weight);
+    table_units(P->pack_items, P->pack_bucket_first, P->grid_blocks, P->pack_small,
+                P->pack_unit_first, P->pack_bucket_unit, pack_weight);
     // Summed weights: a register-path call splits its items over the grid by
     // them (and a bulk launch of a bucket range that gets no pooled slot).
     auto prefix = [](const auto& items, std::vector<unsigned long long>& out, auto w) {

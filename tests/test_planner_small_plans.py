@@ -1,9 +1,10 @@
 """Work tables of small plans: every block gets its work up front.
 
 A plan with less than a 64 KiB item for every block cuts its items so that each
-block has two; a small table's per-bucket units are no more than the grid has
-blocks, and the whole-sync pack's own units hold every item (nothing is left to
-claim).  The tables reproduce the oracle's bytes as any other's.
+block has two; a small table's per-bucket units are fine enough for a range of
+its buckets to give every block some, and the whole-sync pack's own units hold
+every item (nothing is left to claim).  The tables reproduce the oracle's bytes
+as any other's.
 """
 import numpy as np
 import pytest
@@ -30,11 +31,10 @@ def test_small_plan_tables(name, grid):
     assert uitems["nbytes"].max() <= (min(64 * 1024, share) if small else 64 * 1024)
     U.check_units(plan, len(items), "pack")
     units, _ = U.check_units(plan, len(uitems))
+    assert not small or len(units) - 1 >= min(len(uitems), grid)
     full, _ = plan.export_pack_full()
     whole, _ = U.check_units(plan, len(full), "pack_full")
     if small:
-        if len(uitems) < 8 * grid and plan.n_buckets <= grid // 2:
-            assert len(units) - 1 <= grid
         assert whole[grid] == len(full), "a claimed unit holds items"
     shards = L.host_shards(desc["seed"], desc["specials"])
     want, _ = L.pack(oracle.Source(shards=shards))
@@ -60,3 +60,22 @@ def test_small_tables_are_told_by_their_traffic(mi):
     assert small == (mi < 26)
     own = whole[grid] / len(full)
     assert own == 1 if small else 0.8 < own < 0.9
+
+
+@pytest.mark.parametrize("mi,dtype", [(2, "f32"), (4, "bf16"), (12, "f32"), (16, "bf16")])
+def test_ranges_of_small_tables_have_units_for_every_block(mi, dtype):
+    """A range of a small table's buckets: a unit for every block of the grid, or
+    one for every item where there are fewer items."""
+    n, grid = mi << 20, 152
+    plan = rr.rr_plan_create([rr.Param("a", (n,), dtype)], rr.SrcLayout(1),
+                             rr.DstLayout(1, [rr.DstTensor("t", 0, [rr.Block(0, 0, n, 0, 1)])]),
+                             1 << 18, rr.PlanOptions(host_only=True, grid_blocks=grid))
+    for which, items in zip(("pack", "unpack"), (plan.export_pack()[0], plan.export_unpack()[0])):
+        U.check_units(plan, len(items), which)
+        first, bucket_unit = plan.work_units(which)
+        for part in (2, 4, 8):
+            b0 = plan.n_buckets // 4
+            b1 = b0 + plan.n_buckets // part
+            u0, u1 = int(bucket_unit[b0]), int(bucket_unit[b1])
+            n_items = int(first[u1]) - int(first[u0])
+            assert u1 - u0 >= min(n_items, grid), (which, part)
