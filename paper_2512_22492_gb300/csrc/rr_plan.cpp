@@ -55,6 +55,14 @@ constexpr int64_t kSmallPlanItems = 2;         // items per block of a small pla
 // 20 us of a 30 us pack; weighed so, that pack takes 10 us.  The two-layer test
 // model's: 9.3, 9.3, 7.9, 7.4 and 7.6 us with 1, 8, 16, 32 and 64 KiB, its
 // verifying unpack 8.5, 6.5, 6.3 and 6.3 us with 1, 8, 16 and 32 KiB.
+// A pack table of RR_FEW_ITEMS_PER_BLOCK items a block and more keeps its
+// producers busier: there an item weighs its bytes, but at least 32 KiB (1000
+// tensors of 2048 elements and one of 12 M: 21.6 us so, 20.6 with the sum, 35.4
+// with 1 KiB; 1000 of 8192 and one of 8 M: 21.9, 23.9 and 21.6), and where short
+// items share stages 3 KiB more, as on large plans (4000 tensors of 512 elements
+// and one of 4 M: 11.7 us, 22.8 with 32 KiB).  In an unpack table every item has
+// a stage of its own, and the sum holds at any count (3000 tensors of 256
+// elements and one of 4 M: 11.3 us, 19.8 with 1 KiB from eight items a block on).
 #ifndef RR_FEW_ITEMS_OVERHEAD
 #define RR_FEW_ITEMS_OVERHEAD (32 * 1024)
 #endif
@@ -433,18 +441,23 @@ private:
 struct PackWeight {
     bool staged;
     int64_t overhead = kItemOverhead;
+    int64_t least = 0;   // an item's least weight
     int64_t operator()(const rr_pack_item& it) const {
+        return it.kind == RR_ITEM_FAN_DST ? 0 : std::max(least, traffic(it) + overhead);
+    }
+
+private:
+    int64_t traffic(const rr_pack_item& it) const {
         const int64_t n = int64_t(it.row_len) * it.n_rows;
         const int64_t f = !staged ? 20 : it.n_rows > 1 ? 15 : 11;   // tenths of a vector item
         switch (it.kind) {
-            case RR_ITEM_F32_VEC: return 6 * n + overhead;
-            case RR_ITEM_F32_SCALAR: return 6 * n * f / 10 + overhead;
-            case RR_ITEM_BF16_VEC: return 4 * n + overhead;
-            case RR_ITEM_BF16_SCALAR: return 4 * n * f / 10 + overhead;
-            case RR_ITEM_FAN_F32: return 6 * n + overhead;
-            case RR_ITEM_FAN_BF16: return 4 * n + overhead;
-            case RR_ITEM_FAN_DST: return 0;
-            default: return kZeroWeight * n + overhead;
+            case RR_ITEM_F32_VEC: return 6 * n;
+            case RR_ITEM_F32_SCALAR: return 6 * n * f / 10;
+            case RR_ITEM_BF16_VEC: return 4 * n;
+            case RR_ITEM_BF16_SCALAR: return 4 * n * f / 10;
+            case RR_ITEM_FAN_F32: return 6 * n;
+            case RR_ITEM_FAN_BF16: return 4 * n;
+            default: return kZeroWeight * n;
         }
     }
 };
@@ -602,7 +615,7 @@ int64_t unit_weight_for(const std::vector<Item>& items, int32_t grid, W w) {
 // range of buckets can give every block an equal run of them.  As few units as
 // blocks, claimed, left most of the grid idle: packing a 16th of the buckets of a
 // 12 M element fp32 plan took 16.4 us on GB300, and half of them 17.9; with these
-// 7.2 and 13.0.  Of 3, 4, 6, 8 and 16 a block 6 had the fewest ranges slower than
+// 7.2 and 13.5.  Of 3, 4, 6, 8 and 16 a block 6 had the fewest ranges slower than
 // claimed units of at least 128 KiB (coarse runs leave some blocks one unit more,
 // fine ones cut items of unequal weights).
 template <class Item, class W>
@@ -954,17 +967,15 @@ void build_tables(rr_plan* P, const rr_dst_layout* dst) {
         data_bytes < std::min<int64_t>(RR_SHORT_ITEM, P->chunk_bytes / 4) * data_items;
     if (staged && short_items) pack_weight.overhead = RR_SHORT_ITEM_OVERHEAD;
     // Whether a table is small is decided once, on the weights from before the
-    // raise below.
-    auto few = [](const auto& items, int32_t grid) {
-        return int64_t(items.size()) < RR_FEW_ITEMS_PER_BLOCK * int64_t(grid);
-    };
+    // raises below.
     const PackWeight traffic = pack_weight;
+    const bool few = int64_t(P->pack_items.size()) < RR_FEW_ITEMS_PER_BLOCK * int64_t(P->grid_blocks);
     P->pack_small = small_table(total_weight(P->pack_items, traffic), P->grid_blocks,
-                                kSmallPackShare) && few(P->pack_items, P->grid_blocks);
+                                kSmallPackShare) && (few || !short_items);
     P->unpack_small = small_table(total_weight(P->unpack_items, unpack_weight),
-                                  P->unpack_grid_blocks, kSmallUnitShare) &&
-                      few(P->unpack_items, P->unpack_grid_blocks);
-    if (staged && P->pack_small) pack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
+                                  P->unpack_grid_blocks, kSmallUnitShare);
+    if (staged && P->pack_small)
+        (few ? pack_weight.overhead : pack_weight.least) = RR_FEW_ITEMS_OVERHEAD;
     if (staged && P->unpack_small) unpack_weight.overhead = RR_FEW_ITEMS_OVERHEAD;
     P->pack_plain = !short_items;
     P->unpack_plain = true;

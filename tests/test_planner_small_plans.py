@@ -79,3 +79,22 @@ def test_ranges_of_small_tables_have_units_for_every_block(mi, dtype):
             u0, u1 = int(bucket_unit[b0]), int(bucket_unit[b1])
             n_items = int(first[u1]) - int(first[u0])
             assert u1 - u0 >= min(n_items, grid), (which, part)
+
+
+@pytest.mark.parametrize("k,n,mi,dtype,pack_most,unpack_most",
+                         [(1000, 2048, 12, "f32", 24, 16), (1500, 2048, 12, "bf16", 24, 16),
+                          (3000, 256, 4, "f32", 64, 8), (3900, 512, 4, "f32", 64, 8)])
+def test_short_items_of_small_tables_are_spread(k, n, mi, dtype, pack_most, unpack_most):
+    """Many short tensors beside a large one: no block gets a long run of short
+    items, each of which costs it about as much as 32 KiB of traffic.  (Where
+    short items make up the pack table several share a stage, and cost less.)"""
+    sizes = [n] * k + [mi << 20]
+    plan = rr.rr_plan_create([rr.Param(f"p{i}", (s,), dtype) for i, s in enumerate(sizes)],
+                             rr.SrcLayout(1),
+                             rr.DstLayout(1, [rr.DstTensor(f"t{i}", 0, [rr.Block(i, 0, s, 0, 1)])
+                                              for i, s in enumerate(sizes)]),
+                             1 << 20, rr.PlanOptions(host_only=True, grid_blocks=152))
+    whole, _ = U.check_units(plan, len(plan.export_pack_full()[0]), "pack_full")
+    assert np.diff(whole[:153]).max() <= pack_most
+    units, _ = U.check_units(plan, len(plan.export_unpack()[0]))
+    assert np.diff(units).max() <= unpack_most
