@@ -34,7 +34,6 @@ thread_local std::string g_error;
 
 constexpr int64_t kDefaultChunkBytes = 64 * 1024;
 constexpr int64_t kMinChunkBytes = 4 * 1024;   // smallest items of a small plan
-constexpr int64_t kSmallPlanItems = 2;         // items per block of a small plan
 // Balancing weights (build-time overridable for tuning sweeps).  Beyond its
 // bytes an item costs its copies' issue, by one producer warp.  Where short
 // items make up the table (a relay's pieces of 1 to 3 KiB; on average under
@@ -118,12 +117,21 @@ bool is_pow2(int64_t x) { return x > 0 && (x & (x - 1)) == 0; }
 // with three to four of 8 KiB, 14.1 with six to seven of 4 KiB, and 12.2 with
 // 64 KiB items for every other block; pack and verifying unpack of 1, 2 and 4 M
 // elements in turn 11.0, 11.9 and 14.7 us, with 64 KiB items 15.6, 16.1 and
-// 16.9).
-int64_t small_chunk(const rr_plan* P, int32_t grid) {
+// 16.9).  The register path moves one item after the other: there the unpack
+// items of an RR_ENGINE_REGISTERS plan give every block one (verifying unpacks of
+// 0.75 to 8 M elements 8.4 to 10.9 us, with two 8.5 to 11.9, with 64 KiB items
+// 8.7 to 12.6).  Its packs keep two (elements of any alignment go one by one:
+// an odd-sized 2 M pack 15.3 us, with one item a block 19.8, with 64 KiB 32.7).
+// Host buffers on a default plan take the register path over the bulk engine's
+// items: many tensors gain by small ones (an unpack of 65 from pinned buckets
+// 41.4 -> 16.5 us), and a plain pack of 0.25 to 3 MB to or from the host takes up
+// to 1.9 us more than with 64 KiB items (2 MB 17.0 -> 18.6 us).
+int64_t small_chunk(const rr_plan* P, int32_t grid, int items_per_block) {
+    const int64_t items = items_per_block * int64_t(std::max(1, grid));
     int64_t total = 0;
     for (int64_t b : P->rank_stream_bytes) total += b;
     if (total >= P->chunk_bytes * std::max(1, grid)) return P->chunk_bytes;
-    const int64_t share = align_up(total / (kSmallPlanItems * std::max(1, grid)) + 1, 1024);
+    const int64_t share = align_up(total / items + 1, 1024);
     return std::min(P->chunk_bytes, std::max(kMinChunkBytes, share));
 }
 
@@ -1137,8 +1145,8 @@ rr_status rr_plan_create_ex(const rr_param* manifest, int32_t n_params,
                     P->reg_unpack_grid = P->reg_vunpack_grid = opts->grid_blocks;
             P->unpack_chunk_bytes = P->chunk_bytes;
             if (!(opts && opts->chunk_bytes)) {
-                P->chunk_bytes = small_chunk(P, P->grid_blocks);
-                P->unpack_chunk_bytes = small_chunk(P, P->unpack_grid_blocks);
+                P->unpack_chunk_bytes = small_chunk(P, P->unpack_grid_blocks, bulk ? 2 : 1);
+                P->chunk_bytes = small_chunk(P, P->grid_blocks, 2);
             }
         }
         if (st == RR_OK) {

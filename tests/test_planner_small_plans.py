@@ -98,3 +98,23 @@ def test_short_items_of_small_tables_are_spread(k, n, mi, dtype, pack_most, unpa
     assert np.diff(whole[:153]).max() <= pack_most
     units, _ = U.check_units(plan, len(plan.export_unpack()[0]))
     assert np.diff(units).max() <= unpack_most
+
+
+@pytest.mark.parametrize("n", [100_000, 1 << 20, 3_000_001, 8 << 20])
+@pytest.mark.parametrize("engine", ["auto", "registers"])
+def test_items_per_block_of_either_engine(n, engine):
+    """Two items a block, and for the register path's unpacks, which move one item
+    after the other, one."""
+    grid = 304
+    plan = rr.rr_plan_create([rr.Param("a", (n,), "f32")], rr.SrcLayout(1),
+                             rr.DstLayout(1, [rr.DstTensor("t", 0, [rr.Block(0, 0, n, 0, 1)])]),
+                             1 << 20, rr.PlanOptions(host_only=True, grid_blocks=grid,
+                                                     engine=engine))
+    total = sum(plan.stream_bytes_per_rank)
+
+    def share(blocks):
+        return max(4096, min(65536, -(-(total // blocks + 1) // 1024) * 1024))
+
+    assert 2 * int(plan.export_pack()[0]["row_len"].max()) == share(2 * grid)
+    assert int(plan.export_unpack()[0]["nbytes"].max()) == \
+        share(2 * grid if engine == "auto" else grid)
