@@ -29,6 +29,7 @@
 #include <climits>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "rr_internal.h"
 
@@ -62,9 +63,13 @@ namespace {
 #endif
 constexpr int kThreads = RR_THREADS;   // threads per block: pack, plain unpack, verify
 constexpr int kUnroll = RR_UNROLL;     // 16-byte vectors in flight per thread
-// Pointer-table sizes of the two launch shapes.  The small one's parameters fit
-// 4 KB: a launch with 32 KB of them takes 3 us more of host time (the blocking
-// receive of a TP=4 test model, 76 tensors, 27.9 -> 25.2 us).
+// Pointer-table sizes of the launch shapes.  The small one's parameters fit 4
+// KB: a launch with 32 KB of them takes 3 us more of host time (the blocking
+// receive of a TP=4 test model, 76 tensors, 27.9 -> 25.2 us).  The register
+// path's launches, which do not overlap the kernel before them, also show 4 KB
+// against half a KB (a 128 K element pack into pinned buckets 11.6 and 10.6 us):
+// they have the least one as well.
+constexpr int kLeastPtrs = 64;
 constexpr int kSmallPtrs = 448;
 constexpr int kLargePtrs = 3968;    // keeps the kernel parameters under 32 KB
 constexpr int64_t kVerifyChunk = 64 * 1024;
@@ -2056,6 +2061,15 @@ int32_t take_slot(rr_plan* M, cudaStream_t s, LaunchEnd* end);
 template <int MODE, class Args>
 void set_units(const rr_plan* P, const Range& R, Args& a, const uint32_t** first);
 
+// Calls `launch` with the least pointer table (an integral constant) that holds
+// `need` entries: a register-path launch.
+template <class F>
+rr_status with_ptrs(int32_t need, F launch) {
+    if (need <= kLeastPtrs) return launch(std::integral_constant<int, kLeastPtrs>());
+    if (need <= kSmallPtrs) return launch(std::integral_constant<int, kSmallPtrs>());
+    return launch(std::integral_constant<int, kLargePtrs>());
+}
+
 // The register-path pack instantiation for a launch: item checks, a source in
 // host memory, and the destination type.
 template <int NPTR, bool F16>
@@ -2543,11 +2557,10 @@ rr_status pack_impl(const rr_plan* P, Range R, const void* const* src_shards, vo
                                                   nullptr, checksums, nullptr, table, stride, stream,
                                                   o);
         else
-            st = need <= kSmallPtrs
-                     ? launch_pack<kSmallPtrs>(P, S, src_shards, buckets, checksums, table, stride,
-                                               !src_device, stream)
-                     : launch_pack<kLargePtrs>(P, S, src_shards, buckets, checksums, table, stride,
-                                               !src_device, stream);
+            st = with_ptrs(need, [&](auto n) {
+                return launch_pack<decltype(n)::value>(P, S, src_shards, buckets, checksums, table,
+                                                       stride, !src_device, stream);
+            });
         if (st) return st;
     }
     return RR_OK;
@@ -2620,9 +2633,9 @@ rr_status launch_unpack_part(const rr_plan* P, const Range& S, bool bulk,
                              const void* const* buckets, void* const* dst,
                              const uint64_t* checksums, uint8_t* bad, const UnpackShape& sh,
                              cudaStream_t stream, const BulkOpts& o = BulkOpts()) {
-    const bool few = (S.t_hi - S.t_lo + 1) + (sh.table ? S.b1 - S.b0 : 0) <= kSmallPtrs;
+    const int32_t need = (S.t_hi - S.t_lo + 1) + (sh.table ? S.b1 - S.b0 : 0);
     if (bulk) {
-        const bool small = few && !P->check_items;
+        const bool small = need <= kSmallPtrs && !P->check_items;
         if (checksums)
             return small ? launch_bulk<kSmallPtrs, 2>(P, S, nullptr, buckets, dst, checksums, bad,
                                                       sh.table, sh.stride, stream, o)
@@ -2637,10 +2650,10 @@ rr_status launch_unpack_part(const rr_plan* P, const Range& S, bool bulk,
     // the register grid.
     Range Sr = S;
     Sr.full = S.full && P->engine == RR_ENGINE_REGISTERS;
-    return few ? launch_unpack<kSmallPtrs>(P, Sr, buckets, dst, checksums, bad, sh.table,
-                                             sh.stride, stream, o.result, o.result_err)
-                 : launch_unpack<kLargePtrs>(P, Sr, buckets, dst, checksums, bad, sh.table,
-                                             sh.stride, stream, o.result, o.result_err);
+    return with_ptrs(need, [&](auto n) {
+        return launch_unpack<decltype(n)::value>(P, Sr, buckets, dst, checksums, bad, sh.table,
+                                                 sh.stride, stream, o.result, o.result_err);
+    });
 }
 
 rr_status unpack_impl(const rr_plan* P, Range R, const void* const* buckets, void* const* dst,
@@ -2807,11 +2820,10 @@ rr_status verify_impl(const rr_plan* P, Range R, const void* const* buckets,
             RR_CUDA(cudaMemsetAsync(P->d_verify_scratch + n, 0, sizeof(unsigned long long), stream));
         const Range S{b, e, false, nullptr, 0, -1, R.b0, n};
         long long* result = e == R.b1 ? (long long*)P->h_verify_result : nullptr;
-        st = (!table || e - b <= kSmallPtrs)
-                 ? launch_verify<kSmallPtrs>(P, S, buckets, checksums, bad, table, stride, stream,
-                                             one, result)
-                 : launch_verify<kLargePtrs>(P, S, buckets, checksums, bad, table, stride, stream,
-                                             one, result);
+        st = with_ptrs(table ? e - b : 0, [&](auto k) {
+            return launch_verify<decltype(k)::value>(P, S, buckets, checksums, bad, table, stride,
+                                                     stream, one, result);
+        });
         if (st) return st;
     }
     return read_result(P, n_bad, first_bad, stream);
@@ -3244,11 +3256,10 @@ extern "C" rr_status rr_verify_noalloc(const void* const* buckets, int32_t n_buc
     // The array keeps the previous call's contents: clear the sums and counters used here.
     RR_CUDA(cudaMemsetAsync(scratch, 0, (size_t(n_buckets) + 4) * sizeof(unsigned long long),
                             stream));
-    st = (!table || n_buckets <= kSmallPtrs)
-             ? launch_static_verify<kSmallPtrs>(scratch, grid, n_buckets, bucket_bytes, buckets,
-                                                checksums, table, stride, stream)
-             : launch_static_verify<kLargePtrs>(scratch, grid, n_buckets, bucket_bytes, buckets,
-                                                checksums, table, stride, stream);
+    st = with_ptrs(table ? n_buckets : 0, [&](auto k) {
+        return launch_static_verify<decltype(k)::value>(scratch, grid, n_buckets, bucket_bytes,
+                                                        buckets, checksums, table, stride, stream);
+    });
     if (st) return st;
     unsigned long long result[4] = {0, 0, 0, 0};   // host stack: no pinned buffer needed
     RR_CUDA(cudaMemcpyAsync(result, scratch + n_buckets, sizeof result, cudaMemcpyDeviceToHost,
