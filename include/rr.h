@@ -48,8 +48,8 @@
  * instead be host memory this GPU reads (pinned, or any host memory on a
  * device with pageable memory access, as on Grace); memory it cannot reach
  * is refused with RR_EINVAL before anything is launched.  The plan owns its device segment tables,
- * a small verify scratch area and 16 work-unit counters (rr_plan_work_units);
- * rr_pack and rr_unpack allocate nothing.
+ * a small verify scratch area, 16 slots of launch scratch and a stream of its own
+ * (rr_plan_work_units); rr_pack and rr_unpack allocate nothing.
  *
  * Errors.  Every call returns rr_status.  Argument and layout errors are
  * reported synchronously and leave outputs untouched; RR_ECUDA means a CUDA
@@ -59,7 +59,7 @@
  * Threads and streams.  A plan's tables are immutable after creation; rr_pack
  * and rr_unpack may run on it concurrently on different streams, and from
  * different threads, as long as their outputs are distinct (each launch
- * takes its own work-unit counter, under a lock).  rr_verify serialises on
+ * takes its own slot of scratch, under a lock).  rr_verify serialises on
  * the plan.  The stream-ordered calls (rr_pack(_range), rr_unpack(_range),
  * rr_clear_range, rr_unpack_verify_async) may be captured into a CUDA graph;
  * the blocking ones (rr_verify(_range), rr_unpack_verify(_range),
@@ -485,12 +485,14 @@ rr_status rr_plan_bucket_items(const rr_plan* plan, uint32_t* pack_first, uint32
  * caller's for rr_unpack_verify_async) or in a pooled slot; rr_unpack (either
  * engine) and rr_pack (bulk-copy engine) when they get one of the plan's 16
  * pooled slots, as the blocking verifies do.  A stream's launches use the
- * slot that its last one held; another stream takes an idle one, whose last
- * launch has ended.  A launch gets no slot when every slot is held by another
- * stream's launch still in flight, or when its stream is capturing a graph; it
- * then splits its items evenly over the grid, as the register path's pack
- * always does.  Which of these runs changes no output
- * byte. */
+ * slot that its last one held; another stream takes one whose last launch has
+ * ended.  When the host knows of none, the call copies the slots' state from the
+ * device and waits for that (about 10 us; 200 us at most, and no more than a
+ * 20th of the time while it finds none).  A launch gets no slot when every slot
+ * is held by another stream's launch still in flight (or that state could not be
+ * had so), or when its stream is capturing a graph; it then splits its items
+ * evenly over the grid, as the register path's pack always does.  Which of these
+ * runs changes no output byte. */
 enum { RR_UNITS_PACK = 0, RR_UNITS_PACK_FULL = 1, RR_UNITS_UNPACK = 2 };
 rr_status rr_plan_work_units(const rr_plan* plan, int32_t which, int32_t* n_units,
                              uint32_t* unit_first, uint32_t* bucket_unit);

@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <chrono>
 #include <climits>
 #include <cstring>
 #include <mutex>
@@ -2237,24 +2238,53 @@ rr_status launch_verify(const rr_plan* P, Range R, const void* const* buckets,
     return RR_OK;
 }
 
+// Brings the done words to the host, for a call that knows of no idle slot; true
+// when they are there.  The copy runs on a stream of the plan's own and takes
+// about 10 us; the call gives it kDoneWaitUs.  While every slot is in flight such
+// waits find nothing: after one, calls only start the copy, for those after
+// them, until kDoneWaitShare times its length has passed.  (With copies for later
+// calls alone, seventeen streams in turn left one without a slot for good: the
+// other sixteen had launched again whenever it looked.)
+constexpr int kDoneWaitUs = 200, kDoneWaitShare = 20;
+bool refresh_done(rr_plan* M) {
+    using Clock = std::chrono::steady_clock;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // another thread may capture
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const Clock::time_point t0 = Clock::now();
+    if (cudaStreamQuery(M->slot_copies) == cudaSuccess)   // else the last copy is under way
+        cudaMemcpyAsync(M->h_slot_done, M->d_slot_done,
+                        rr_plan::kClaimSlots * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                        M->slot_copies);
+    bool here = false;
+    if (t0 >= M->next_done_wait) {
+        while (!(here = cudaStreamQuery(M->slot_copies) == cudaSuccess) &&
+               Clock::now() - t0 < std::chrono::microseconds(kDoneWaitUs)) {
+        }
+        M->next_done_wait = Clock::now() + kDoneWaitShare * (Clock::now() - t0);
+    }
+    cudaGetLastError();   // cudaErrorNotReady, of a copy under way
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return here;
+}
+
 // A pooled slot for a launch on `s`, or -1; fills in *end for it.  The slot that
 // the stream's own last launch held serves again: a stream runs its launches
 // in order, so that one is done with it first (a bulk kernel touches its slot
 // only past griddepcontrol.wait).  Otherwise one that no launch has held yet,
 // or whose last launch is known to have ended: each launch leaves its number
-// in a device word, and a call that finds no slot has these words copied to
-// the host, on a stream of the plan's own, for the calls after it.  So a launch
-// costs its slot neither an event (about 1 us each to record and to query, and
-// one between two kernels keeps the second from starting its prologue under
-// the first's tail) nor a store to host memory (2 us at the end of a 10 us
-// kernel).  There is none when every slot is, as far as known, held by another
-// stream's launch, or when `s` is capturing a graph (a captured launch replays
-// whenever the graph does).  The caller holds claim_mutex and sets
-// slot_seq[slot] = end->seq once the launch is enqueued (a launch that failed
-// leaves the slot as it was: zero, its last launch's number in place).  A slot
-// is all zero when handed out: zeroed once at plan creation, then by the last
-// block of each launch that held it.  Streams are told apart by their unique
-// id: a handle may come back for a new stream.
+// in a device word, and a call that knows of no idle slot has these words
+// copied to the host.  So a launch costs its slot neither an event (about 1 us
+// each to record and to query, and one between two kernels keeps the second
+// from starting its prologue under the first's tail) nor a store to host memory
+// (2 us at the end of a 10 us kernel).  There is none when every slot is held by
+// another stream's launch (or is not known to be idle, refresh_done), or when
+// `s` is capturing a graph (a captured launch replays whenever the graph does).
+// The caller holds claim_mutex and sets slot_seq[slot] = end->seq once the launch
+// is enqueued (a launch that failed leaves the slot as it was: zero, its last
+// launch's number in place).  A slot is all zero when handed out: zeroed once at
+// plan creation, then by the last block of each launch that held it.  Streams are told apart by their unique
+// id: a handle may come back for a new stream, and cudaStreamPerThread is
+// another stream, with another id, in every thread.
 int32_t take_slot(rr_plan* M, cudaStream_t s, LaunchEnd* end) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     unsigned long long id = 0;
@@ -2267,21 +2297,16 @@ int32_t take_slot(rr_plan* M, cudaStream_t s, LaunchEnd* end) {
     int32_t slot = -1;
     for (int32_t k = 0; k < rr_plan::kClaimSlots && slot < 0; ++k)
         if (M->slot_seq[k] != 0 && M->slot_stream[k] == id) slot = k;
-    for (int32_t i = 0; i < rr_plan::kClaimSlots && slot < 0; ++i) {
-        const int32_t k = (M->claim_next + i) % rr_plan::kClaimSlots;
-        if (__atomic_load_n(M->h_slot_done + k, __ATOMIC_ACQUIRE) == M->slot_seq[k]) slot = k;
-    }
-    if (slot < 0) {
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // another thread may capture
-        cudaThreadExchangeStreamCaptureMode(&mode);
-        if ((!M->slot_copies &&
-             cudaStreamCreateWithFlags(&M->slot_copies, cudaStreamNonBlocking) != cudaSuccess) ||
-            cudaMemcpyAsync(M->h_slot_done, M->d_slot_done,
-                            rr_plan::kClaimSlots * sizeof(unsigned long long),
-                            cudaMemcpyDeviceToHost, M->slot_copies) != cudaSuccess)
-            cudaGetLastError();
-        cudaThreadExchangeStreamCaptureMode(&mode);
-        return -1;
+    auto find_idle = [&] {
+        for (int32_t i = 0; i < rr_plan::kClaimSlots && slot < 0; ++i) {
+            const int32_t k = (M->claim_next + i) % rr_plan::kClaimSlots;
+            if (__atomic_load_n(M->h_slot_done + k, __ATOMIC_ACQUIRE) == M->slot_seq[k]) slot = k;
+        }
+        return slot >= 0;
+    };
+    if (slot < 0 && !find_idle()) {
+        if (!refresh_done(M) || !find_idle()) return -1;
+        M->next_done_wait = {};   // a wait that found one: the next may be as useful
     }
     M->claim_next = (slot + 1) % rr_plan::kClaimSlots;
     M->slot_stream[slot] = id;
@@ -2898,12 +2923,12 @@ rr_status rr_device_upload(rr_plan* P) {
                                                  sizeof(unsigned long long))) != cudaSuccess ||
         (e = cudaMemset(P->d_slots, 0, rr_plan::kClaimSlots * (P->slot_words() + 1) *
                                            sizeof(unsigned long long))) != cudaSuccess ||
-
         (e = cudaMalloc((void**)&P->d_verify_scratch,
                         (size_t(P->n_buckets) + 4) * sizeof(unsigned long long))) != cudaSuccess ||
         (e = cudaHostAlloc((void**)&P->h_verify_result,
                            (8 + rr_plan::kClaimSlots) * sizeof(unsigned long long),
                            cudaHostAllocDefault)) != cudaSuccess ||
+        (e = cudaStreamCreateWithFlags(&P->slot_copies, cudaStreamNonBlocking)) != cudaSuccess ||
         (e = cudaMalloc((void**)&P->d_error, sizeof(unsigned int))) != cudaSuccess ||
         (e = cudaMemset(P->d_error, 0, sizeof(unsigned int))) != cudaSuccess ||
         (e = up((void**)&P->d_pack_weight_prefix, P->pack_weight_prefix.data(),

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <atomic>
+#include <chrono>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -121,7 +122,8 @@ struct rr_plan {
     unsigned long long slot_stream[kClaimSlots] = {};  // the id of the last one's stream
     unsigned long long* d_slot_done = nullptr;         // the number of the last that ended,
     unsigned long long* h_slot_done = nullptr;         //   and a pinned copy of some time ago,
-    cudaStream_t slot_copies = nullptr;                //   made on this stream
+    cudaStream_t slot_copies = nullptr;                //   made on this stream, and when a
+    std::chrono::steady_clock::time_point next_done_wait{};   // call may next wait for one
     int32_t claim_next = 0;
     std::mutex claim_mutex;
     std::atomic<uint64_t> prepared{0};   // bulk kernels whose shared memory is set up

@@ -1,17 +1,15 @@
 """Work units claimed at run time by the bulk-copy engine's blocks.
 
 rr_pack and rr_unpack take a slot (a claim counter, and for pack its sums)
-from a pool of 16 per plan.  A slot is free once the launch that last held
-it has completed.  When none is, a launch takes the slot handed out longest
-ago if that slot's launch ran on its own stream, and waits on the GPU for it.
-A launch finds no slot when every slot is held by another stream's launch
-still in flight, or when it is being captured into a CUDA graph.  It then
-zeroes its checksums first and splits its items evenly over the grid.  These
-tests drive every one of those paths and compare bytes with the oracle:
+from a pool of 16 per plan.  A stream's launches hold the slot that its last one
+held, one after another; a stream that has none takes one whose last launch has
+ended.  A launch finds no slot when every slot is held by another stream's
+launch still in flight (tests/test_gpu_launch_slots.py), or when it is being
+captured into a CUDA graph.  It then zeroes its checksums first and splits its
+items evenly over the grid.  These tests compare bytes with the oracle for:
   - more launches in flight on one stream than slots (the stream held back by
     a bounded sleep kernel, so that none of them can complete before the rest
-    are enqueued), and meanwhile a second stream's launches, which find every
-    slot held;
+    are enqueued), all through one slot, and meanwhile a second stream's;
   - two streams packing and unpacking their own buffers at once;
   - the whole step captured into a CUDA graph and replayed on new inputs;
   - a resumed pull's range calls (clear, pack, unpack, stream-ordered check)
@@ -71,11 +69,11 @@ def test_more_launches_in_flight_than_claim_slots():
     other = torch.cuda.Stream()
     torch.cuda.synchronize()
     torch.cuda._sleep(SLEEP_CYCLES)            # nothing below can complete until it ends
-    for b in bufs:                             # past 16, each waits for the oldest slot
+    for b in bufs:                             # one slot for all of them, in stream order
         rr.rr_pack(plan, b.shards, b.buckets, b.checksums)
     for b in bufs:
         rr.rr_unpack(plan, b.buckets, b.dst)
-    for b in side:                             # every slot held by the first stream: none
+    for b in side:                             # and another for this stream's
         rr.rr_pack(plan, b.shards, b.buckets, b.checksums, stream=other)
         rr.rr_unpack(plan, b.buckets, b.dst, stream=other)
     torch.cuda.synchronize()

@@ -1,16 +1,15 @@
 """One plan driven from several host threads at once.
 
 include/rr.h lets a plan run concurrently on different streams, from different
-threads, as long as the outputs are distinct (each launch takes its own
-work-unit counter under the plan's lock; the blocking verify serialises on the
-plan).  Here six threads share one plan and one source; each has its own
-stream, buckets, checksums, tensors, scratch and result rows, and runs many
-steps of rr_pack, the stream-ordered verifying unpack, bucket-range packs and
-the blocking verify, so that launches contend for the plan's 16 counter slots
-(and take the fallbacks when none is free).  Every thread's buckets,
-checksums and tensors must equal the oracle's at the end (RobustRL Section
-5.2.1: many rollouts pull from one trainer; Section 5.2.2: each checks what it
-holds).
+threads, as long as the outputs are distinct (each launch takes its own slot
+under the plan's lock; the blocking verify serialises on the plan).  Here six
+threads share one plan and one source; each has its own stream, buckets,
+checksums, tensors, scratch and result rows, and runs many steps of rr_pack, the
+stream-ordered verifying unpack, bucket-range packs and the blocking verify, so
+that their launches take slots of the plan's pool of 16 at the same time.  Every
+thread's buckets, checksums and tensors must equal the oracle's at the end
+(RobustRL Section 5.2.1: many rollouts pull from one trainer; Section 5.2.2: each
+checks what it holds).
 """
 import os
 import threading
