@@ -479,8 +479,12 @@ def _ptr_array(xs) -> ctypes.Array:
 def _stream(stream) -> int:
     if stream is None:
         import torch
-        # The current stream's handle without a Stream object (3 us on Grace).
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        # The current stream's handle without a Stream object (3 us on Grace),
+        # by the call that torch's own code generators use; it is not public.
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return raw(torch.cuda.current_device())
+        return int(torch.cuda.current_stream().cuda_stream)
     if isinstance(stream, int):
         return stream
     return int(stream.cuda_stream)

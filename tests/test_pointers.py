@@ -152,3 +152,23 @@ def test_pageable_host_buffers_refused_where_unreadable():
     with pytest.raises(rr.RRError) as e:
         rr.rr_verify(plan, buf.buckets, torch.zeros(plan.n_buckets, dtype=torch.int64))
     assert e.value.status == rrmod.RR_EINVAL
+
+
+@pytest.mark.parametrize("raw", [True, False])
+def test_current_stream_with_and_without_torchs_raw_call(monkeypatch, raw):
+    """The current stream's handle does not depend on a private torch call."""
+    from types import SimpleNamespace
+
+    import torch
+    from paper_2512_22492_gb300 import rr as binding
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream",
+                        lambda *a: SimpleNamespace(cuda_stream=0x1230))
+    if raw:
+        monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda d: 0x1230 + d,
+                            raising=False)
+    else:
+        monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    assert binding._stream(None) == (0x1233 if raw else 0x1230)
+    assert binding._stream(7) == 7
+    assert binding._stream(SimpleNamespace(cuda_stream=9)) == 9
