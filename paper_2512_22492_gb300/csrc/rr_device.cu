@@ -19,7 +19,8 @@
 // register path each block takes a contiguous, weight-balanced range of it.
 // On the bulk-copy engine blocks take work units: their own first, then the
 // next unclaimed one (an atomic counter) until none are left, so that blocks
-// draining HBM at unequal rates still finish together.  The work is pure
+// draining HBM at unequal rates still finish together (small tables' blocks take
+// equal runs of units, without claims).  The work is pure
 // data movement bound by HBM bandwidth; the cast is integer arithmetic in
 // registers, and the checksum is accumulated per warp and flushed with one
 // 64-bit atomic per warp per bucket change.
@@ -380,8 +381,8 @@ __device__ __forceinline__ uint32_t lower_item(const unsigned long long* prefix,
     return lo;
 }
 
-// This block's item range: the plan's balanced split for a full call, an even
-// split of [begin, end) for a bucket-range call.
+// This block's item range in a launch without work units: the plan's balanced
+// split for a full call, a split of [begin, end) for a bucket-range call.
 __device__ __forceinline__ void block_items(const uint32_t* block_first,
                                             const unsigned long long* prefix, uint32_t begin,
                                             uint32_t end, uint32_t* i0, uint32_t* i1) {
@@ -832,7 +833,7 @@ __global__ void __launch_bounds__(kThreads, 5) rr_verify_kernel(const __grid_con
 
 // ---------------------------------------------------------------------------
 // Bulk-copy engine (cp.async.bulk + mbarrier), the default for buffers in
-// device memory.  One producer lane per block turns the block's work items
+// device memory.  One producer warp per block turns the block's work items
 // into pieces: long contiguous or row-strided 16-byte-aligned runs are loaded
 // into a ring of shared-memory stages with cp.async.bulk (rows of a strided
 // run land back to back); elements at any other alignment are staged in the
@@ -2020,8 +2021,9 @@ rr_status check_buf(int dev, bool pageable_ok, const void* p, const char* what,
     return RR_OK;
 }
 
-// A call covers buckets [b0, b1).  The full range uses the plan's balanced
-// per-block item ranges; a sub-range splits its items evenly over the grid.
+// A call covers buckets [b0, b1).  full: all of them, in one launch (without work
+// units it uses the plan's balanced per-block item ranges, else it splits its
+// items over the grid by their weights).
 struct Range {
     int32_t b0, b1;
     bool full;
@@ -2357,9 +2359,10 @@ void set_units(const rr_plan* P, const Range& R, Args& a, const uint32_t** first
 
 // How a bulk launch may use the plan's pooled slots, and what it zeroes itself.
 struct BulkOpts {
-    bool may_slot = true;                 // try a pooled slot (not for the blocking verifies)
-    unsigned long long* zero = nullptr;   // without a slot, zero these words first (pack:
-    size_t zero_words = 0;                //   the range's checksums; async verify: scratch)
+    bool may_slot = true;                 // try a pooled slot (a verifying call's only launch,
+                                          //   or one that sums nothing)
+    unsigned long long* zero = nullptr;   // without a slot, zero these words first (pack: the
+    size_t zero_words = 0;                //   range's checksums; verifying unpack: scratch)
     long long* result = nullptr;          // verifying unpack: write {n_bad, first_bad} here
     bool result_err = false;              //   and the plan's error word after them
 };
@@ -2718,11 +2721,11 @@ rr_status read_result(const rr_plan* P, int64_t* n_bad, int64_t* first_bad, cuda
     return h[0] ? RR_EMISMATCH : RR_OK;
 }
 
-// Enqueues the verifying unpack of range R.  The stream-ordered form (R has
-// the caller's scratch) in one bulk launch sums into a pooled slot when one is
-// free, zeroing nothing first; otherwise the range's sums and counters
-// (R.scratch, else the plan's) are zeroed, then one fused launch per sub-range
-// (usually one) runs.  Sub-launches share the call's counters; each compares
+// Enqueues the verifying unpack of range R, whose scratch is the caller's
+// (R.scratch, the stream-ordered form) or the plan's (the blocking one).  One bulk
+// launch sums into a pooled slot when one is free, zeroing nothing first;
+// otherwise the range's sums and counters in the scratch are zeroed, then one
+// fused launch per sub-range (usually one) runs.  Sub-launches share the call's counters; each compares
 // its own buckets, and the "last block" ticket and the unit claims are reset
 // between them.  `result` (device address or NULL) receives {n_bad,
 // first_bad} from the last launch's last block.
@@ -2785,7 +2788,7 @@ rr_status unpack_verify_impl(const rr_plan* P, Range R, const void* const* bucke
     if (n_bad) *n_bad = 0;
     if (first_bad) *first_bad = -1;
     if (R.b1 == R.b0) return RR_OK;
-    rr_plan* M = const_cast<rr_plan*>(P);   // the scratch area is the only mutable state
+    rr_plan* M = const_cast<rr_plan*>(P);   // its scratch, pinned answer and slots are mutable state
     std::lock_guard<std::mutex> lock(M->verify_mutex);
     P->h_verify_result[2] = kNoAnswer;
     if ((st = enqueue_unpack_verify(P, R, buckets, checksums, dst, bad, on_device, stream,
@@ -2794,11 +2797,10 @@ rr_status unpack_verify_impl(const rr_plan* P, Range R, const void* const* bucke
     return read_result(P, n_bad, first_bad, stream);
 }
 
-// {n_bad, first_bad or -1} from a verifying pass's counters (NULL: an empty range).
-__global__ void rr_verify_result_kernel(const unsigned long long* counters, long long* result) {
-    const unsigned long long nb = counters ? counters[1] : 0ull;
-    result[0] = (long long)nb;
-    result[1] = nb ? (long long)(ULLONG_MAX - counters[2]) : -1ll;
+// The stream-ordered result of an empty range.
+__global__ void rr_empty_result_kernel(long long* result) {
+    result[0] = 0;
+    result[1] = -1;
 }
 
 // The device address of a result buffer: device memory, or pinned (mapped)
@@ -2828,7 +2830,7 @@ rr_status verify_impl(const rr_plan* P, Range R, const void* const* buckets,
     uint64_t stride = 0;
     const bool table = !uniform(buckets, P->n_buckets, P->bucket_bytes, &stride);
 
-    rr_plan* M = const_cast<rr_plan*>(P);   // the scratch area is the only mutable state
+    rr_plan* M = const_cast<rr_plan*>(P);   // its scratch, pinned answer and slots are mutable state
     std::lock_guard<std::mutex> lock(M->verify_mutex);
     P->h_verify_result[2] = kNoAnswer;
     const int32_t n = R.b1 - R.b0;
@@ -3118,7 +3120,7 @@ extern "C" rr_status rr_unpack_verify_async(const rr_plan* P, int32_t first_buck
         // The launch's last block writes the result.
         return enqueue_unpack_verify(P, R, buckets, checksums, dst, bad, on_device, stream, res);
     }
-    rr_verify_result_kernel<<<1, 1, 0, stream>>>(nullptr, res);   // an empty range
+    rr_empty_result_kernel<<<1, 1, 0, stream>>>(res);
     RR_CUDA(cudaGetLastError());
     return RR_OK;
 }

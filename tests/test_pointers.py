@@ -159,7 +159,6 @@ def test_current_stream_with_and_without_torchs_raw_call(monkeypatch, raw):
     """The current stream's handle does not depend on a private torch call."""
     from types import SimpleNamespace
 
-    import torch
     from paper_2512_22492_gb300 import rr as binding
     monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
     monkeypatch.setattr(torch.cuda, "current_stream",
