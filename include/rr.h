@@ -195,7 +195,7 @@ typedef struct {
                             a plan can be queried and exported but not executed       */
     int32_t grid_blocks; /* persistent grid size; default: SMs x resident blocks      */
     int64_t chunk_bytes; /* largest destination bytes per work item; default 64 KiB,
-                            on small plans less (down to 8 KiB)                       */
+                            on small plans less (down to 4 KiB)                       */
     int32_t engine;      /* rr_engine                                                 */
     int32_t check_items; /* 1: every kernel checks each work item against the source,
                             bucket and tensor sizes of the plan before touching
@@ -471,6 +471,13 @@ rr_status rr_plan_bucket_items(const rr_plan* plan, uint32_t* pack_first, uint32
  *     units after them cut the rest to the sizes above, smaller toward the
  *     end.  A cut never falls before a fan-out destination item.  Own units
  *     may be empty.
+ *   Small tables (under 1 MiB of traffic a block of the grid for a pack, 256
+ *   KiB for an unpack) are not claimed.  The own shares of a whole pack then
+ *   hold all of the table.  The per-bucket units are all of one size, about six
+ *   a block, and the blocks of a range call take equal runs of its units; an
+ *   unpack over every bucket takes shares of the table, at most one a block.
+ *   (Packs of many short one-row items that share stages keep claimed
+ *   per-bucket units.)
  *   *n_units: the number of units.
  *   unit_first (NULL, or n_units + 1 entries): unit u holds items
  *     [unit_first[u], unit_first[u + 1]) of that table.
