@@ -498,8 +498,9 @@ rr_status rr_plan_bucket_items(const rr_plan* plan, uint32_t* pack_first, uint32
  * 20th of the time while it finds none).  A launch gets no slot when every slot
  * is held by another stream's launch still in flight (or that state could not be
  * had so), or when its stream is capturing a graph; it then splits its items
- * evenly over the grid, as the register path's pack always does.  Which of these
- * runs changes no output byte. */
+ * evenly over the grid, as the register path's pack always does (a range call on
+ * a small table takes its units' equal runs all the same).  Which of these runs
+ * changes no output byte. */
 enum { RR_UNITS_PACK = 0, RR_UNITS_PACK_FULL = 1, RR_UNITS_UNPACK = 2 };
 rr_status rr_plan_work_units(const rr_plan* plan, int32_t which, int32_t* n_units,
                              uint32_t* unit_first, uint32_t* bucket_unit);
@@ -509,7 +510,8 @@ rr_status rr_plan_work_units(const rr_plan* plan, int32_t which, int32_t* n_unit
  * 5.2.2: the pull completes, and a resumed pull checks what it holds).
  *   first_bucket, n_buckets: the range (0 and the plan's count for all).
  *   scratch: caller device memory of n_buckets + 4 uint64, 16-byte aligned;
- *            zeroed and used by the call, free again once `result` is written.
+ *            zeroed and used by the call when it gets no slot (rr_plan_work_units),
+ *            free again once `result` is written.
  *            Calls that overlap in time need distinct scratch.
  *   result:  two int64 in device memory or pinned (mapped) host memory, 8-byte
  *            aligned; when the call's work is done on `stream` they hold
