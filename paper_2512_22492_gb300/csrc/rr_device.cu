@@ -1054,9 +1054,9 @@ __device__ __forceinline__ void gather_async(uint32_t stage, uint32_t full_bar, 
 // These elements used to be read one by one from global memory by the
 // consumers, each load waited for (19.5 of 24 cycles per issue on the load,
 // DRAM at 8%).  Staged, the path is bound by HBM like the aligned one: packing
-// a 274 M-element model of odd sizes (1.65 GB moved) went from 2467 to 250 us
-// on GB300 (243 at the measured copy rate), the verifying unpack of one whose tensors and buckets differ in
-// phase from 2957 to 165 us.  The limit between the two copy forms lies where
+// a 274 M-element model of odd sizes (1.65 GB moved) went from 2467 to 254 us
+// on GB300 (243 at the measured copy rate), the verifying unpack of one whose
+// tensors and buckets differ in phase from 2957 to 165 us.  The limit between the two copy forms lies where
 // they cost the same: a bulk copy takes the copy unit about 35 ns whatever its
 // size, a gather about 35 ns per 512 bytes.  Packs of bf16 rows
 // of 72 bytes run at 660 GB/s by bulk copies and 2280 by gathers, of 514 bytes

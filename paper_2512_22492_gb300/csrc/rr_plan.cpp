@@ -40,8 +40,9 @@ constexpr int64_t kMinChunkBytes = 4 * 1024;   // smallest items of a small plan
 // RR_SHORT_ITEM bytes and a quarter of the plan's largest) that is about 3 KiB
 // of traffic an item: such a relay's pack ran at 430, 371, 338, 287, 273 and 273
 // us with 0, 0.5, 1, 2, 3 and 4 KiB.  Tables of large items with a few short
-// ones among them run the same with each, and the odd-sized one best with 1
-// (244 us, 250 with 3).
+// ones among them run the same with each, and the odd-sized one best with 1 (its
+// pack 244 us against 250 with 3, before the kernels emitted every kind of item
+// in one loop: 254 since).
 #ifndef RR_ITEM_OVERHEAD
 #define RR_ITEM_OVERHEAD 1024
 #endif
