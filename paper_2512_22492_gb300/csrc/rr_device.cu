@@ -1056,11 +1056,11 @@ __device__ __forceinline__ void gather_async(uint32_t stage, uint32_t full_bar, 
 // DRAM at 8%).  Staged, the path is bound by HBM like the aligned one: packing
 // a 274 M-element model of odd sizes (1.65 GB moved) went from 2467 to 254 us
 // on GB300 (243 at the measured copy rate), the verifying unpack of one whose
-// tensors and buckets differ in phase from 2957 to 165 us.  The limit between the two copy forms lies where
-// they cost the same: a bulk copy takes the copy unit about 35 ns whatever its
-// size, a gather about 35 ns per 512 bytes.  Packs of bf16 rows
-// of 72 bytes run at 660 GB/s by bulk copies and 2280 by gathers, of 514 bytes
-// at 3050 and 3620, of 1002 bytes at 4260 and 3430.
+// tensors and buckets differ in phase from 2957 to 165 us.  The limit between the
+// two copy forms lies where they cost the same: a bulk copy takes the copy unit
+// about 35 ns whatever its size, a gather about 35 ns per 512 bytes.  Packs of
+// bf16 rows of 72 bytes run at 660 GB/s by bulk copies and 2280 by gathers, of 514
+// bytes at 3050 and 3620, of 1002 bytes at 4260 and 3430.
 __device__ __forceinline__ uint32_t rag_pitch(uint32_t row_len, uint32_t es) {
     return (row_len * es + 31 - es) & ~15u;   // the widest window: shift 16 - es
 }
@@ -2283,9 +2283,9 @@ bool refresh_done(rr_plan* M) {
 // The caller holds claim_mutex and sets slot_seq[slot] = end->seq once the launch
 // is enqueued (a launch that failed leaves the slot as it was: zero, its last
 // launch's number in place).  A slot is all zero when handed out: zeroed once at
-// plan creation, then by the last block of each launch that held it.  Streams are told apart by their unique
-// id: a handle may come back for a new stream, and cudaStreamPerThread is
-// another stream, with another id, in every thread.
+// plan creation, then by the last block of each launch that held it.  Streams are
+// told apart by their unique id: a handle may come back for a new stream, and
+// cudaStreamPerThread is another stream, with another id, in every thread.
 int32_t take_slot(rr_plan* M, cudaStream_t s, LaunchEnd* end) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     unsigned long long id = 0;
@@ -2727,10 +2727,10 @@ rr_status read_result(const rr_plan* P, int64_t* n_bad, int64_t* first_bad, cuda
 // (R.scratch, the stream-ordered form) or the plan's (the blocking one).  One bulk
 // launch sums into a pooled slot when one is free, zeroing nothing first;
 // otherwise the range's sums and counters in the scratch are zeroed, then one
-// fused launch per sub-range (usually one) runs.  Sub-launches share the call's counters; each compares
-// its own buckets, and the "last block" ticket and the unit claims are reset
-// between them.  `result` (device address or NULL) receives {n_bad,
-// first_bad} from the last launch's last block.
+// fused launch per sub-range (usually one) runs.  Sub-launches share the call's
+// counters; each compares its own buckets, and the "last block" ticket and the
+// unit claims are reset between them.  `result` (device address or NULL) receives
+// {n_bad, first_bad} from the last launch's last block.
 rr_status enqueue_unpack_verify(const rr_plan* P, Range R, const void* const* buckets,
                                 const uint64_t* checksums, void* const* dst, uint8_t* bad,
                                 bool on_device, cudaStream_t stream, long long* result) {
@@ -2790,7 +2790,7 @@ rr_status unpack_verify_impl(const rr_plan* P, Range R, const void* const* bucke
     if (n_bad) *n_bad = 0;
     if (first_bad) *first_bad = -1;
     if (R.b1 == R.b0) return RR_OK;
-    rr_plan* M = const_cast<rr_plan*>(P);   // its scratch, pinned answer and slots are mutable state
+    rr_plan* M = const_cast<rr_plan*>(P);   // its scratch, answer and slots are mutable
     std::lock_guard<std::mutex> lock(M->verify_mutex);
     P->h_verify_result[2] = kNoAnswer;
     if ((st = enqueue_unpack_verify(P, R, buckets, checksums, dst, bad, on_device, stream,
@@ -2832,7 +2832,7 @@ rr_status verify_impl(const rr_plan* P, Range R, const void* const* buckets,
     uint64_t stride = 0;
     const bool table = !uniform(buckets, P->n_buckets, P->bucket_bytes, &stride);
 
-    rr_plan* M = const_cast<rr_plan*>(P);   // its scratch, pinned answer and slots are mutable state
+    rr_plan* M = const_cast<rr_plan*>(P);   // its scratch, answer and slots are mutable
     std::lock_guard<std::mutex> lock(M->verify_mutex);
     P->h_verify_result[2] = kNoAnswer;
     const int32_t n = R.b1 - R.b0;
