@@ -2955,6 +2955,9 @@ rr_status rr_device_upload(rr_plan* P) {
     P->h_slot_done = P->h_verify_result + 8;
     std::memset(P->h_verify_result, 0,
                 (8 + rr_plan::kClaimSlots) * sizeof(unsigned long long));
+    // The copies above may return before their data has arrived, and the plan's
+    // launches may run on streams that do not wait for the default one.
+    RR_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     return RR_OK;
 }
 
